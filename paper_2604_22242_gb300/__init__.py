@@ -13,6 +13,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import threading
 
 __all__ = [
     "FxError", "FX_F32", "FX_F64", "FX_BF16", "FX_F16", "FX_MAX_SLOTS", "lib", "lib_path",
@@ -280,8 +281,32 @@ def bind_tensor(h, slot: int, t):
     fx_expr_bind(h, slot, t.data_ptr(), rows, cols, ld)
 
 
+# Handles whose last launches may still be running when their owner lets go
+# of them: (event recorded after those launches, handle). fx_expr_destroy
+# frees workspace without waiting for the kernels that use it, so a handle is
+# destroyed only once its event has completed; at most _RETIRED_MAX are held.
+_retired = []
+_retired_lock = threading.Lock()
+_RETIRED_MAX = 32
+
+
+def _retire(event, h):
+    with _retired_lock:
+        _retired.append((event, h))
+        done = [e for e in _retired if e[0].query()]
+        _retired[:] = [e for e in _retired if e not in done]
+        while len(_retired) > _RETIRED_MAX:
+            e = _retired.pop(0)
+            e[0].synchronize()
+            done.append(e)
+    for _, x in done:
+        fx_expr_destroy(x)
+
+
 class Expr:
     """An expression object with its slots bound to torch tensors."""
+
+    _last = None  # event after the last launches; set where nobody else waits for them
 
     def __init__(self, name: str, storage: int):
         self.h = fx_expr_create(name, storage)
@@ -306,10 +331,19 @@ class Expr:
     def eval_unfused(self, stream=None):
         fx_eval_unfused(self.h, _stream_ptr(stream))
 
+    def mark(self):
+        """Notes that launches of this handle are in flight on the current
+        stream: close() then destroys it only after they have finished."""
+        self._last = _torch().cuda.Event()
+        self._last.record()
+
     def close(self):
         if self.h:
-            fx_expr_destroy(self.h)
-            self.h = None
+            h, self.h = self.h, None
+            if self._last is None:
+                fx_expr_destroy(h)
+            else:
+                _retire(self._last, h)
 
     def __del__(self):
         try:
@@ -340,6 +374,7 @@ def FusedLoss():
             out = torch.empty((1, 1), dtype=rdt, device=inputs[0].device)
             ex.bind(ex.n_in, out)
             ex.eval()
+            ex.mark()  # the graph, and this handle with it, may go before the kernels end
             ctx.ex = ex
             ctx.save_for_backward(*inputs)
             return out.reshape(())
@@ -357,6 +392,7 @@ def FusedLoss():
             gl = gL.to(torch.float64 if ex.storage == FX_F64 else torch.float32).reshape(1).contiguous()
             fx_eval_backward(ex.h, gl.data_ptr(), [g.data_ptr() for g in grads],
                              _stream_ptr(None))
+            ex.mark()
             ctx.keep = gl
             return (None, None, *grads)
 
