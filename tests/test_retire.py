@@ -51,5 +51,5 @@ def test_busy_handle_waits_for_its_event(destroyed):
 def test_held_handles_are_bounded(destroyed):
     events = [Event() for _ in range(fx._RETIRED_MAX + 3)]
     for k, e in enumerate(events):
-        handle(k, e).close()
-    assert destroyed == [0, 1, 2] and [e.waits for e in events[:4]] == [1, 1, 1, 0]
+        handle(k + 1, e).close()
+    assert destroyed == [1, 2, 3] and [e.waits for e in events[:4]] == [1, 1, 1, 0]
