@@ -23,6 +23,7 @@
 #include <cmath>
 
 #include "core.cuh"
+#include "dmath.cuh"
 
 namespace fx {
 
@@ -38,11 +39,16 @@ FX_HD constexpr int flip_mode(int m) {
 // used by the fused backward pass (k_bwd, k_bwd_bulk).
 
 FX_D float m_exp(float x) { return ::expf(x); }
-FX_D double m_exp(double x) { return ::exp(x); }
+FX_D double m_exp(double x) { return dm::exp_fast_ok(x) ? dm::exp_fast(x) : dm::exp_any(x); }
 FX_D float m_log(float x) { return ::logf(x); }
 FX_D double m_log(double x) { return ::log(x); }
 FX_D float m_sqrt(float x) { return ::sqrtf(x); }
-FX_D double m_sqrt(double x) { return ::sqrt(x); }
+FX_D double m_sqrt(double x) { return dm::sqrt_fast_ok(x) ? dm::sqrt_fast(x) : dm::sqrt_any(x); }
+// Division: FP32 by the operator; FP64 by dmath.cuh
+FX_D float m_div(float a, float b) { return a / b; }
+FX_D double m_div(double a, double b) {
+  return dm::div_fast_ok(a, b) ? dm::div_fast(a, b) : dm::div_any(a, b);
+}
 FX_D float m_abs(float x) { return ::fabsf(x); }
 FX_D double m_abs(double x) { return ::fabs(x); }
 FX_D float m_tanh(float x) { return ::tanhf(x); }
@@ -60,17 +66,17 @@ template <class C> FX_D C m_gt(C a, C b) { return a > b ? C(1) : C(0); }
 // plus |x| * 2^-23 relative from scaling x by log2(e), is further damped by
 // the factor 1 - sigmoid in the result), exp for FP64.
 FX_D float m_exp_sig(float x) { return __expf(x); }
-FX_D double m_exp_sig(double x) { return ::exp(x); }
+FX_D double m_exp_sig(double x) { return m_exp(x); }
 // The reciprocal inside sigmoid: the hardware's approximate reciprocal for
 // FP32 (one instruction, within about one ulp; its argument 1 + exp(-x) is
-// at least 1, so flushing subnormals changes nothing), the correctly
-// rounded one for FP64.
+// at least 1, so flushing subnormals changes nothing), the FP64
+// division of dmath.cuh for FP64.
 FX_D float m_rcp_sig(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-FX_D double m_rcp_sig(double x) { return __drcp_rn(x); }
+FX_D double m_rcp_sig(double x) { return m_div(1.0, x); }
 
 // ---------------------------------------------------------------- lane pairs
 //
@@ -117,7 +123,7 @@ FX_D F2 m_fma(F2 a, F2 b, F2 c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)), "l"(f2_bits(c)));
   return f2_of(r);
 }
-FX_D F2 operator/(F2 a, F2 b) { return F2(a.x / b.x, a.y / b.y); }
+FX_D F2 m_div(F2 a, F2 b) { return F2(a.x / b.x, a.y / b.y); }
 FX_D F2 operator-(F2 a) { return F2(-a.x, -a.y); }
 FX_D F2& operator+=(F2& a, F2 b) { return a = a + b; }
 // equal in both lanes (used on broadcast scalars)
@@ -147,10 +153,10 @@ struct OpMul {
   template <class C> static FX_D void d(C a, C b, C& da, C& db) { da = b; db = a; }
 };
 struct OpDiv {
-  template <class C> static FX_D C f(C a, C b) { return a / b; }
+  template <class C> static FX_D C f(C a, C b) { return m_div(a, b); }
   template <class C> static FX_D void d(C a, C b, C& da, C& db) {
     da = m_rcp(b);
-    db = -a / (b * b);
+    db = m_div(-a, b * b);
   }
 };
 struct OpPow {  // a ^ b (b is a scalar in the trees built here; 2 and 3 by multiplication)
@@ -203,11 +209,11 @@ struct OpExp {
 };
 struct OpLog {
   template <class C> static FX_D C f(C a) { return m_log(a); }
-  template <class C> static FX_D C d(C a, C) { return C(1) / a; }
+  template <class C> static FX_D C d(C a, C) { return m_div(C(1), a); }
 };
 struct OpSqrt {
   template <class C> static FX_D C f(C a) { return m_sqrt(a); }
-  template <class C> static FX_D C d(C, C z) { return C(0.5) / z; }
+  template <class C> static FX_D C d(C, C z) { return m_div(C(0.5), z); }
 };
 struct OpAbs {
   template <class C> static FX_D C f(C a) { return m_abs(a); }
