@@ -7,6 +7,7 @@
 #include <string>
 
 
+#include "skew.cuh"
 #include "tmatile.cuh"
 #include "runtime.hpp"
 
@@ -461,8 +462,33 @@ fx_status launch_tile_tma(const Run& r, const E& e, const Slots& sl, int64_t R, 
   }
 }
 
+// k_tile_skew; *used is false when the plain leaves and Z do not share
+// their misalignment (or the leaves are of several types).
+template <class T, class E, class EpiV, class Epi1, int V>
+fx_status launch_tile_skew(const Run& r, const E& e, const Slots& sl, int64_t R, int64_t C,
+                           const EpiV& ev, const Epi1& e1, RedArgs red, bool* used) {
+  using LL = leaves_t<E>;
+  *used = false;
+  if constexpr (V > 1 && V * sizeof(T) == 16 && tma_uniform<LL, T>()) {
+    const void* z = nullptr;
+    if constexpr (EpiV::stores) z = ev.z;
+    uint32_t sbase = 0, sld = 0;
+    if (!skew_ok<LL, T, V>(r.b, z, ev.ldz, sbase, sld)) return FX_OK;
+    using TC_ = TileCfg<E, V>;
+    auto kern = k_tile_skew<E, EpiV, Epi1, T, V, TC_::TR, TC_::TC, TC_::NT>;
+    const int64_t ntiles = ((R + V - 1 + TC_::TR - 1) / TC_::TR) * ((C + TC_::TC - 1) / TC_::TC);
+    const int grid = grid_for(kern, TC_::NT, ntiles > 0 ? ntiles : 1, r.tune);
+    if constexpr (EpiV::reduces) FX_TRY(red_space(r, grid, red));
+    *used = true;
+    kern<<<grid, TC_::NT, 0, r.st>>>(e, sl, R, C, ev, e1, red, sbase, sld);
+    return after_launch(r, "k_tile_skew");
+  }
+  return FX_OK;
+}
+
 // Tiles of a tree with transposed leaves. Launch-shape pipeline 0: the
-// TMA kernel when the operands allow it; 1: the cp.async pipeline when
+// TMA kernel when the operands allow it, else (unless aligned vectors do)
+// the skewed tiles when the operands share their misalignment; 1: the cp.async pipeline when
 // every plain leaf and the output are vector-aligned; otherwise, and for
 // pipeline 2, the register-staged kernel.
 template <class T, class E, class EpiV, class Epi1, int V>
@@ -474,6 +500,10 @@ fx_status launch_tiles(const Run& r, const E& e, const Slots& sl, int64_t R, int
       bool used = false;
       const fx_status s = launch_tile_tma<T>(r, e, sl, R, C, ev, red, &used);
       if (s != FX_OK || used) return s;
+      if (!vec) {
+        const fx_status k = launch_tile_skew<T, E, EpiV, Epi1, V>(r, e, sl, R, C, ev, e1, red, &used);
+        if (k != FX_OK || used) return k;
+      }
     }
   }
   if constexpr (count_mt<LL>() > 0 && V > 1 && TileAsyncCfg<E, V>::SMEM <= 200 * 1024) {
