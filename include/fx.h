@@ -250,7 +250,8 @@ fx_status fx_expr_set_launch_shape(fx_expr* x, int block, int unroll, int blocks
                                    int pipeline);
 
 /* Number of kernel launches the last evaluation call on this object
- * enqueued (for launch accounting). */
+ * enqueued (for launch accounting). Counts launches that evaluate the tree;
+ * library GEMMs and launches that lay out a product's operands are not in it. */
 int fx_expr_last_launches(const fx_expr* x);
 
 /* Synchronises `stream`, then reports FX_E_CUDA if an asynchronous CUDA

@@ -16,9 +16,12 @@
 // chain Z = A * B * C * D).
 #pragma once
 
+#include <initializer_list>
+
 #include <cublas_v2.h>
 
 #include "umma.cuh"
+#include "umma32.cuh"
 #include "unfused.cuh"
 
 namespace fx {
@@ -277,12 +280,12 @@ template <class L, class R> struct ScaledProd<SL<OpMul, Prod<L, R>>> {
 
 // ---------------------------------------------------------------- tcgen05 path
 
-// Trees the tensor-core kernel takes: BF16 or FP16 storage, one matrix
+// Trees the tensor-core kernels take: BF16, FP16 or FP32 storage, one matrix
 // product of two matrix leaves (plain or transposed), and an element-wise
 // remainder whose other leaves are plain matrices of the storage type.
 template <class T, int NIN, class Root> struct umma_ok {
   static constexpr bool value = [] {
-    if constexpr (!(std::is_same<T, bf16>::value || std::is_same<T, f16>::value)) {
+    if constexpr (std::is_same<T, double>::value) {
       return false;
     } else if constexpr (root_of<Root>::kind != FX_KIND_ELEMENTWISE || !has_prod_v<Root>) {
       return false;
@@ -353,6 +356,104 @@ fx_status run_umma(fx_expr* x, const Root& root, cudaStream_t st, bool* used) {
   return FX_OK;
 }
 
+// Do two bound matrices of `es`-byte elements share memory (as whole spans)?
+inline bool overlap(const Binding& x, const Binding& y, size_t es) {
+  auto span = [es](const Binding& b) { return (size_t(b.ld) * size_t(b.cols - 1) + size_t(b.rows)) * es; };
+  const uintptr_t p = reinterpret_cast<uintptr_t>(x.p), q = reinterpret_cast<uintptr_t>(y.p);
+  return p < q + span(y) && q < p + span(x);
+}
+
+// FP32: the operands split into BF16 planes, then umma32::k_gemm_umma32 (two
+// launches). Takes operands of any alignment and leading dimension, since
+// the planes are laid out here. *used is false when the shapes disagree (the
+// library path reports it), an extent is beyond the kernels' indices, or
+// the workspace for the planes cannot be had (the library path needs less).
+template <int NIN, class Root>
+fx_status run_umma32(fx_expr* x, const Root& root, cudaStream_t st, bool* used) {
+  namespace u3 = umma32;
+  *used = false;
+  using LR = Lift<Root, float, NIN>;
+  using Lifted = typename LR::type;
+  constexpr int PS = NIN;
+  using P = typename the_prod<Root>::type;
+  using OA = Operand<std::decay_t<decltype(std::declval<P>().l)>>;
+  using OB = Operand<std::decay_t<decltype(std::declval<P>().r)>>;
+  constexpr bool AMN = !OA::trans, BMN = OB::trans;
+  const Binding& a = x->b[OA::slot];
+  const Binding& b = x->b[OB::slot];
+  const Binding& zb = x->b[NIN];
+  if (!a.bound || !b.bound || !zb.bound) return FX_OK;
+  const int64_t M = OA::trans ? a.cols : a.rows, K = OA::trans ? a.rows : a.cols;
+  const int64_t Kb = OB::trans ? b.cols : b.rows, N = OB::trans ? b.rows : b.cols;
+  if (K != Kb || zb.rows != M || zb.cols != N || M == 0 || N == 0 || K == 0) return FX_OK;
+  const int64_t lim = int64_t(1) << 30;
+  if (M >= lim || N >= lim || K >= lim) return FX_OK;
+  // Z written over an operand: the fallback for unsplittable values reads the
+  // operands while other blocks store
+  if (overlap(zb, a, sizeof(float)) || overlap(zb, b, sizeof(float))) return FX_OK;
+  const int64_t ntiles = ((M + u3::BM - 1) / u3::BM) * ((N + u3::BN - 1) / u3::BN);
+  const int64_t pieces = (int64_t(1) << 32) - 1;
+  auto items = [](const Binding& o) { return (o.rows + 7) / 8 * o.cols; };
+  if (ntiles >= (int64_t(1) << 26) || items(a) > pieces || items(b) > pieces) return FX_OK;
+  Binding bt[FX_MAX_SLOTS];
+  for (int k = 0; k < NIN; ++k) bt[k] = x->b[k];
+  bt[PS] = Binding{nullptr, M, N, M, true};
+  if (check_leaves<leaves_t<Lifted>>(bt, M, N) != FX_OK) {
+    cudaGetLastError();
+    return FX_OK;
+  }
+  const int sms = device_sms() > 0 ? device_sms() : 1;
+  const int S = u3::choose_splits(ntiles, int((K + u3::BK - 1) / u3::BK), sms);
+  auto up = [](size_t v) { return (v + 255) & ~size_t(255); };
+  auto ldp = [](const Binding& o) { return (o.rows + 7) / 8 * 8; };
+  const size_t pa = up(size_t(ldp(a)) * size_t(a.cols) * 6), pb = up(size_t(ldp(b)) * size_t(b.cols) * 6);
+  const size_t pp = S > 1 ? size_t(ntiles) * S * u3::BM * u3::BN * sizeof(float) : 0;
+  if (x->ws_gemm.ensure(pa + pb + pp, st) != FX_OK) {
+    cudaGetLastError();
+    return FX_OK;
+  }
+  const Run r = run_of(x, st);
+  unsigned int *tick = nullptr, *err = nullptr;
+  FX_TRY(tickets(r, ntiles + 2, &tick));
+  FX_TRY(err_word(r, &err));
+  bf16* da = static_cast<bf16*>(x->ws_gemm.p);
+  bf16* db = da + pa / 2;
+  float* part = reinterpret_cast<float*>(db + pb / 2);
+  u3::Maps maps;
+  auto planes = [&](const Binding& o, bf16* d, int box1, std::initializer_list<int> at) {
+    int64_t p = 0;
+    for (int k : at)
+      if (!encode_map<bf16>(&maps.m[k], d + p++ * ldp(o) * o.cols, o.rows, o.cols, ldp(o), 64, box1))
+        return false;
+    return true;
+  };
+  if (!planes(a, da, AMN ? 64 : u3::BM, {u3::A1, u3::A2, u3::A3}) ||
+      !planes(b, db, BMN ? 64 : u3::BN, {u3::B1, u3::B2, u3::B3}))
+    return FX_OK;
+  auto split = [&](const Binding& o, bf16* d) {
+    return u3::SplitArgs{static_cast<const float*>(o.p), d, o.rows, o.cols, o.ld, ldp(o), items(o),
+                         FastDiv::make(uint32_t((o.rows + 7) / 8)),
+                         aligned(o.p, 16) && o.ld % 4 == 0 ? 1 : 0};
+  };
+  auto kern = u3::k_gemm_umma32<AMN, BMN, Lifted, PS>;
+  const int smem = 2 * u3::NP * u3::TILE + 1024 + int(sizeof(u3::Bars));
+  FX_TRY(allow_smem(kern, smem));
+  *used = true;
+  x->last_launches = 0;
+  const int64_t blocks = (items(a) + items(b) + 255) / 256;
+  u3::k_split3<<<unsigned(blocks < sms * 8 ? blocks : sms * 8), 256, 0, st>>>(split(a, da), split(b, db),
+                                                                              tick);
+  FX_TRY(after_launch(r, "k_split3"));
+  x->last_launches = 0;  // counts launches that evaluate the tree, not those that lay out operands
+  const int64_t nitems = ntiles * S;
+  const u3::Source sa{static_cast<const float*>(a.p), AMN ? 1 : a.ld, AMN ? a.ld : 1};
+  const u3::Source sb{static_cast<const float*>(b.p), BMN ? 1 : b.ld, BMN ? b.ld : 1};
+  kern<<<unsigned(nitems < sms ? nitems : sms), u3::THREADS, smem, st>>>(
+      maps, LR::make(root), make_slots(x->b, NIN), static_cast<float*>(zb.p), zb.ld, int(M), int(N),
+      int(K), S, part, tick + 2, tick, sa, sb, err);
+  return after_launch(r, "k_gemm_umma32");
+}
+
 // A tree with matrix products: products into temporaries (slots NIN ..
 // NIN+P-1 of a private binding table), then the lifted tree on the fused
 // path (or, for the unfused baseline, one launch per operator).
@@ -369,7 +470,12 @@ fx_status run_with_prods(fx_expr* x, const Root& root, int kind, cudaStream_t st
     // its epilogue; 1 and 2: the library GEMM and the fused pass
     if (!unfused && kind == FX_KIND_ELEMENTWISE && x->tune.pipe == 0) {
       bool used = false;
-      FX_TRY((run_umma<T, NIN>(x, root, st, &used)));
+      if constexpr (!std::is_same<T, float>::value) {
+        FX_TRY((run_umma<T, NIN>(x, root, st, &used)));
+      } else if constexpr (!ScaledProd<Root>::value) {
+        // a bare or scaled FP32 product has nothing to fuse: the library GEMM
+        FX_TRY((run_umma32<NIN>(x, root, st, &used)));
+      }
       if (used) return FX_OK;
     }
   }

@@ -137,9 +137,14 @@ template <class LL, int PS, class T, int CW> struct ECtx {
   }
 };
 
-// An ordered 2-byte load (volatile, memory clobber): the epilogue's loads
+// An ordered load (volatile, memory clobber): the epilogue's loads
 // of the next chunk are issued before the current chunk is computed and
 // stored, and the compiler may not sink them next to their use.
+FX_D float ld_ordered(const float* p) {
+  float v;
+  asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
 template <class TL> FX_D TL ld_ordered(const TL* p) {
   static_assert(sizeof(TL) == 2, "16-bit leaves");
   unsigned short v;
