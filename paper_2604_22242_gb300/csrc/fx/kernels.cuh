@@ -12,7 +12,7 @@
 // (s, c) pair over a fixed set of elements; warps and blocks combine pairs
 // in a fixed butterfly order; each block writes one partial; the last block
 // to finish (an atomic ticket, no waiting) sums the partials in a fixed
-// order in FP64 and writes the result. No block ever waits on another.
+// order as pairs and writes the result. No block ever waits on another.
 #pragma once
 
 #include "plan.cuh"
@@ -465,22 +465,66 @@ template <class CT> FX_D CT block_max(CT m) {
   return m;
 }
 
-// Fixed-order FP64 sum of n partial pairs part[i*stride]; the result is
-// valid in thread 0. Every thread of the block must call it. COMP selects
-// a compensated sum (FP64 trees, whose 1e-13 bound needs it); for FP32
-// trees a plain FP64 sum of the partials is already about 2^-40 relative,
-// and FP64 operations are scarce on this part.
-template <bool COMP> FX_D double block_sum_partials(const double2* part, int64_t n, int64_t stride) {
-  using S = std::conditional_t<COMP, CompSum<double>, PlainSum<double>>;
-  S a;
+// A published partial sum: the pair (s, c) in the compute type. The
+// combines add pairs as pairs (CompSum): for FP64 trees a compensated FP64
+// sum, for FP32 trees one that carries about 48 bits. Summing FP32 trees'
+// partials in FP64 instead would be no closer after the final rounding to
+// FP32, and this part issues a warp-wide FP64 add in about 64 cycles: the
+// last block of an 8192-row backward range spent 19 us on its 78k adds
+// while the other SMs were idle. Forward and backward of the 8192 x 8192 BF16
+// loss: 218 us with FP64 combines, 199 us with these.
+template <class CT> struct pair_of { using type = float2; };
+template <> struct pair_of<double> { using type = double2; };
+template <class CT> using pair_t = typename pair_of<CT>::type;
+template <class CT> FX_D pair_t<CT> make_pair_of(CT s, CT c) {
+  pair_t<CT> q;
+  q.x = s;
+  q.y = c;
+  return q;
+}
+template <class CT> FX_D pair_t<CT>* pairs(double2* part) {
+  return reinterpret_cast<pair_t<CT>*>(part);
+}
+
+// An FP32 pair sum that left FP32's range on the way (partials that cancel
+// beyond it, or an infinite total) is taken again in FP64.
+FX_D bool redo_in_f64(float s) { return !(fabsf(s) <= 3.4028234663852886e38f); }
+FX_D bool redo_in_f64(double) { return false; }
+
+// Sum of the n pairs part[k * stride] of one row, by one thread, in FP64.
+template <class CT> FX_D CT sum_pairs_f64(const pair_t<CT>* part, int64_t n, int64_t stride) {
+  double a = 0.0;
+  for (int64_t k = 0; k < n; ++k) {
+    const pair_t<CT> q = __ldcg(part + k * stride);
+    a = a + double(q.x) + double(q.y);
+  }
+  return CT(a);
+}
+
+// Fixed-order sum of n partial pairs, in FP64 after the pairs' merge; the
+// result is valid in thread 0. Every thread of the block must call it.
+template <class CT> FX_D double block_sum_partials(const pair_t<CT>* part, int64_t n) {
+  CompSum<CT> a;
   a.init();
   for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-    double2 q = __ldcg(part + i * stride);
-    a.add(q.x);
-    a.add(q.y);
+    const pair_t<CT> q = __ldcg(part + i);
+    a.merge(q.x, q.y);
   }
   block_merge(a);
-  return a.s + a.c;
+  if constexpr (!std::is_same<CT, double>::value) {
+    if (__syncthreads_or(threadIdx.x == 0 && redo_in_f64(a.s))) {
+      PlainSum<double> d;
+      d.init();
+      for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
+        const pair_t<CT> q = __ldcg(part + i);
+        d.add(double(q.x));
+        d.add(double(q.y));
+      }
+      block_merge(d);
+      return d.s;
+    }
+  }
+  return double(a.s) + double(a.c);
 }
 
 // Every block publishes its partial; the last one combines all of them.
@@ -488,7 +532,7 @@ template <class CT, bool SQRT, class S> FX_D void finish_full_reduce(S& a, const
   block_merge(a);
   __shared__ bool last;
   if (threadIdx.x == 0) {
-    red.part[blockIdx.x] = make_double2(double(a.s), double(a.c));
+    pairs<CT>(red.part)[blockIdx.x] = make_pair_of<CT>(a.s, a.c);
     __threadfence();
     unsigned int t = atomicAdd(red.ticket, 1u);
     last = (t == gridDim.x - 1);
@@ -496,7 +540,7 @@ template <class CT, bool SQRT, class S> FX_D void finish_full_reduce(S& a, const
   __syncthreads();
   if (!last) return;
   __threadfence();
-  double tot = block_sum_partials<std::is_same<CT, double>::value>(red.part, gridDim.x, 1);
+  double tot = block_sum_partials<CT>(pairs<CT>(red.part), gridDim.x);
   if (threadIdx.x == 0) {
     if (SQRT) tot = ::sqrt(tot);
     *static_cast<CT*>(red.out) = static_cast<CT>(tot);
@@ -862,14 +906,14 @@ __global__ void __launch_bounds__(NT) k_col(const E e, const Slots sl, const int
         res = warp_max(m);
       } else {
         warp_merge(acc);
-        res = CT(double(acc.s) + double(acc.c));
+        res = add_rn(acc.s, acc.c);
       }
     } else {
       if (ISMAX) {
         res = block_max(m);
       } else {
         block_merge(acc);
-        res = CT(double(acc.s) + double(acc.c));
+        res = add_rn(acc.s, acc.c);
       }
     }
     if (lane == 0 && c < C) static_cast<CT*>(out)[c * ldo] = res;
@@ -901,14 +945,14 @@ FX_D void row_finish(const RowRed& rr, ThreadSum<CT> (&acc)[V], CT (&m)[V], int6
   if (rr.S == 1) {
 #pragma unroll
     for (int j = 0; j < V; ++j)
-      if (j < nvalid) out[r + j] = ISMAX ? m[j] : CT(double(acc[j].s) + double(acc[j].c));
+      if (j < nvalid) out[r + j] = ISMAX ? m[j] : add_rn(acc[j].s, acc[j].c);
     return;
   }
 #pragma unroll
   for (int j = 0; j < V; ++j) {
     if (j < nvalid) {
       if (ISMAX) static_cast<CT*>(rr.partm)[int64_t(s) * R + r + j] = m[j];
-      else rr.part[int64_t(s) * R + r + j] = make_double2(double(acc[j].s), double(acc[j].c));
+      else pairs<CT>(rr.part)[int64_t(s) * R + r + j] = make_pair_of<CT>(acc[j].s, acc[j].c);
     }
   }
   __threadfence();
@@ -948,37 +992,35 @@ FX_D void row_finish(const RowRed& rr, ThreadSum<CT> (&acc)[V], CT (&m)[V], int6
     for (int j = 0; j < V; ++j)
       if (j < nvalid) out[r + j] = mm[j];
   } else {
-    using S = std::conditional_t<std::is_same<CT, double>::value, CompSum<double>, PlainSum<double>>;
-    S a[V];
+    const pair_t<CT>* part = pairs<CT>(rr.part);
+    CompSum<CT> a[V];
 #pragma unroll
     for (int j = 0; j < V; ++j) a[j].init();
     int k = 0;
     for (; k + KU <= rr.S; k += KU) {
-      double2 q[KU][V];
+      pair_t<CT> q[KU][V];
 #pragma unroll
       for (int t = 0; t < KU; ++t)
 #pragma unroll
         for (int j = 0; j < V; ++j)
-          q[t][j] = j < nvalid ? __ldcg(rr.part + int64_t(k + t) * R + r + j) : make_double2(0, 0);
+          q[t][j] = j < nvalid ? __ldcg(part + int64_t(k + t) * R + r + j) : make_pair_of<CT>(0, 0);
 #pragma unroll
       for (int t = 0; t < KU; ++t)
 #pragma unroll
-        for (int j = 0; j < V; ++j) {
-          a[j].add(q[t][j].x);
-          a[j].add(q[t][j].y);
-        }
+        for (int j = 0; j < V; ++j) a[j].merge(q[t][j].x, q[t][j].y);
     }
     for (; k < rr.S; ++k)
 #pragma unroll
       for (int j = 0; j < V; ++j)
         if (j < nvalid) {
-          double2 q = __ldcg(rr.part + int64_t(k) * R + r + j);
-          a[j].add(q.x);
-          a[j].add(q.y);
+          const pair_t<CT> q = __ldcg(part + int64_t(k) * R + r + j);
+          a[j].merge(q.x, q.y);
         }
 #pragma unroll
     for (int j = 0; j < V; ++j)
-      if (j < nvalid) out[r + j] = CT(a[j].s + a[j].c);
+      if (j < nvalid)
+        out[r + j] = redo_in_f64(a[j].s) ? sum_pairs_f64<CT>(part + r + j, rr.S, R)
+                                         : add_rn(a[j].s, a[j].c);
   }
   if (threadIdx.x == 0) rr.tickets[blockIdx.x] = 0u;
 }
@@ -1139,7 +1181,10 @@ FX_D void bwd_store(const GradAcc<LL, CT, E> (&g)[V], CT (&bpart)[NB][V],
 }
 
 // Last block of a row range: sum the column splits' row partials in split
-// order (FP64, compensated) and write each_col leaves' gradients (dense).
+// order (as pairs) and write each_col leaves' gradients (dense). A split's
+// pairs of a thread's V rows are loaded for KU splits before any is added:
+// only one block per row range is at work here, so the loads' latency, not
+// their number, is what the tail of the launch waits for.
 template <class LL, int V, class CT, int I = 0>
 FX_D void bwd_bc_finish(const GradArgs& ga, int64_t r, int64_t R, int nvalid) {
   if constexpr (I < tl_size<LL>::value) {
@@ -1149,19 +1194,30 @@ FX_D void bwd_bc_finish(const GradArgs& ga, int64_t r, int64_t R, int nvalid) {
       constexpr int b = bc_rank<LL, I>();
       T* dst = static_cast<T*>(ga.g[L::slot]);
       if (dst) {
+        constexpr int KU = 8;
+        const pair_t<CT>* part = pairs<CT>(ga.part) + int64_t(b) * ga.S * R + r;
+        CompSum<CT> a[V];
 #pragma unroll
-        for (int j = 0; j < V; ++j) {
-          if (j < nvalid) {
-            std::conditional_t<std::is_same<CT, double>::value, CompSum<double>, PlainSum<double>> a;
-            a.init();
-            for (int k = 0; k < ga.S; ++k) {
-              double2 q = __ldcg(ga.part + (int64_t(b) * ga.S + k) * R + r + j);
-              a.add(q.x);
-              a.add(q.y);
-            }
-            sstore(dst + r + j, narrow_to<T>::from(CT(a.s + a.c)));
-          }
+        for (int j = 0; j < V; ++j) a[j].init();
+        for (int k = 0; k < ga.S; k += KU) {
+          pair_t<CT> q[KU][V];
+#pragma unroll
+          for (int t = 0; t < KU; ++t)
+#pragma unroll
+            for (int j = 0; j < V; ++j)
+              q[t][j] = (k + t < ga.S && j < nvalid) ? __ldcg(part + int64_t(k + t) * R + j)
+                                                     : make_pair_of<CT>(0, 0);
+#pragma unroll
+          for (int t = 0; t < KU; ++t)
+#pragma unroll
+            for (int j = 0; j < V; ++j) a[j].merge(q[t][j].x, q[t][j].y);
         }
+#pragma unroll
+        for (int j = 0; j < V; ++j)
+          if (j < nvalid)
+            sstore(dst + r + j,
+                   narrow_to<T>::from(redo_in_f64(a[j].s) ? sum_pairs_f64<CT>(part + j, ga.S, R)
+                                                          : CT(add_rn(a[j].s, a[j].c))));
       }
     }
     bwd_bc_finish<LL, V, CT, I + 1>(ga, r, R, nvalid);
@@ -1180,8 +1236,8 @@ FX_D void bwd_finish(const GradArgs& ga, ThreadSum<CT> (&bacc)[NB][V], int64_t R
 #pragma unroll
       for (int j = 0; j < V; ++j)
         if (j < nvalid)
-          ga.part[(int64_t(b) * ga.S + s) * R + r + j] =
-              make_double2(double(bacc[b][j].s), double(bacc[b][j].c));
+          pairs<CT>(ga.part)[(int64_t(b) * ga.S + s) * R + r + j] =
+              make_pair_of<CT>(bacc[b][j].s, bacc[b][j].c);
     __threadfence();
     block_sync(nthreads);
     if (abort && *abort) return;  // a bounded wait gave up (recorded); no combine
