@@ -20,8 +20,8 @@
 //   div   3 FP64 instructions, the same way from the FP32 reciprocal.
 //
 // X % Y + sqrt(abs(W)) / (1 + exp(-V)) needs 12 FP64 instructions an element
-// this way and 35 with CUDA's functions; at 3001 x 4096 the four statistics
-// calls of which it is the first went from 1156 to 682 us.
+// this way and 35 with CUDA's functions: 0.28 ms at 3001 x 4096, where FP64
+// sign changes (expr.cuh) took it to 14 and 0.34 ms.
 //
 // The last step of sqrt and div adds a correction of relative size 2^-45 with
 // a relative error below 2^-20 to it, so the result is the correctly

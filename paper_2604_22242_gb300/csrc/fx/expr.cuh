@@ -50,7 +50,11 @@ FX_D double m_div(double a, double b) {
   return dm::div_fast_ok(a, b) ? dm::div_fast(a, b) : dm::div_any(a, b);
 }
 FX_D float m_abs(float x) { return ::fabsf(x); }
-FX_D double m_abs(double x) { return ::fabs(x); }
+// FP64 sign changes by integer instructions: as FP64 ones they would run at
+// the scarce unit's rate (dmath.cuh).
+FX_D double m_abs(double x) { return dm::from_words(dm::hi_word(x) & 0x7FFFFFFFu, dm::lo_word(x)); }
+template <class C> FX_D C m_neg(C x) { return -x; }
+FX_D double m_neg(double x) { return dm::from_words(dm::hi_word(x) ^ 0x80000000u, dm::lo_word(x)); }
 FX_D float m_tanh(float x) { return ::tanhf(x); }
 FX_D double m_tanh(double x) { return ::tanh(x); }
 // 1 / x correctly rounded (the same value as the IEEE division 1 / x,
@@ -200,7 +204,7 @@ template <int S, class CT> FX_D CT lin_adj(CT adj) {
 }
 
 struct OpNeg {
-  template <class C> static FX_D C f(C a) { return -a; }
+  template <class C> static FX_D C f(C a) { return m_neg(a); }
   template <class C> static FX_D C d(C, C) { return C(-1); }
 };
 struct OpExp {
@@ -224,7 +228,7 @@ struct OpSquare {
   template <class C> static FX_D C d(C a, C) { return C(2) * a; }
 };
 struct OpSigmoid {  // Sec. 4: sigmoid = 1 / (1 + exp(-X))
-  template <class C> static FX_D C f(C a) { return m_rcp_sig(C(1) + m_exp_sig(-a)); }
+  template <class C> static FX_D C f(C a) { return m_rcp_sig(C(1) + m_exp_sig(m_neg(a))); }
   template <class C> static FX_D C d(C, C z) { return z * (C(1) - z); }
 };
 struct OpTanh {

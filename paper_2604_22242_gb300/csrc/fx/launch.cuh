@@ -77,12 +77,15 @@ template <class K> fx_status allow_smem(K kern, int bytes) {
   return FX_OK;
 }
 
-// Column splits for row-range kernels: enough blocks for the resident
-// capacity, at least 2*minc columns per split.
+// Column splits for row-range kernels: as many blocks as are resident at
+// once, at least 2*minc columns per split. Rounded down: a few blocks more
+// than are resident run after all others, for as long as those did (FP64
+// maxima of the rows of 3001 x 4096: 312 blocks on 304 places took 169 us,
+// 300 take 96 us).
 inline int64_t row_splits(int64_t gx, int64_t C, int occ, int minc, const Tune& t) {
   const int sms = device_sms() > 0 ? device_sms() : 1;
   const int bps = t.bps > 0 ? (t.bps < occ ? t.bps : occ) : occ;
-  int64_t S = (int64_t(sms) * (bps > 0 ? bps : 1) + gx - 1) / gx;
+  int64_t S = int64_t(sms) * (bps > 0 ? bps : 1) / (gx > 0 ? gx : 1);
   const int64_t smax = C / (2 * minc) > 1 ? C / (2 * minc) : 1;
   if (S > smax) S = smax;
   if (S > 65535) S = 65535;
@@ -639,7 +642,13 @@ template <class E, int D> struct dim_of<MaxDim<E, D>> { static constexpr int d =
 template <class E, bool ISMAX, int V>
 fx_status launch_col(const Run& r, const E& e, const Slots& sl, int64_t R, int64_t C, void* out,
                      int64_t ldo) {
-  constexpr int NT = 256, U = tl_size<leaves_t<E>>::value <= 2 ? 8 : 4;
+  // a warp's loads in flight cover latency with U vectors; FP64 takes fewer,
+  // so that more warps (columns) fit on an SM
+  constexpr int NT = 256, U = !std::is_same<ct_of<E>, double>::value && tl_size<leaves_t<E>>::value <= 2 ? 8 : 4;
+  // blocks of two warps when a warp takes a column: with eight, the columns
+  // of 4096 filled the SMs unevenly (one round and an eighth). FP64 column
+  // sums of 3001 x 4096: 95 us with U = 8 and eight warps, 49 us so
+  constexpr int NW = 64;
   // a block per column for long FP32 columns; a warp per column otherwise,
   // and for FP64 up to 2^16 rows: its slow FP64 unit leaves a block per
   // column waiting on the block-wide merge after only a few steps
@@ -649,10 +658,10 @@ fx_status launch_col(const Run& r, const E& e, const Slots& sl, int64_t R, int64
     const int grid = grid_for(kern, NT, C > 0 ? C : 1, r.tune);
     kern<<<grid, NT, 0, r.st>>>(e, sl, R, C, out, ldo);
   } else {
-    auto kern = k_col<E, ISMAX, V, U, 32, NT>;
-    const int64_t work = (C + NT / 32 - 1) / (NT / 32);
-    const int grid = grid_for(kern, NT, work > 0 ? work : 1, r.tune);
-    kern<<<grid, NT, 0, r.st>>>(e, sl, R, C, out, ldo);
+    auto kern = k_col<E, ISMAX, V, U, 32, NW>;
+    const int64_t work = (C + NW / 32 - 1) / (NW / 32);
+    const int grid = grid_for(kern, NW, work > 0 ? work : 1, r.tune);
+    kern<<<grid, NW, 0, r.st>>>(e, sl, R, C, out, ldo);
   }
   return after_launch(r, "k_col");
 }
