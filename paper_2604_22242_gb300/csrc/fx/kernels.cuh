@@ -530,6 +530,14 @@ template <class CT> FX_D double block_sum_partials(const pair_t<CT>* part, int64
 // Every block publishes its partial; the last one combines all of them.
 template <class CT, bool SQRT, class S> FX_D void finish_full_reduce(S& a, const RedArgs& red) {
   block_merge(a);
+  if (gridDim.x == 1) {  // nothing to combine
+    if (threadIdx.x == 0) {
+      double tot = double(a.s) + double(a.c);
+      if (SQRT) tot = ::sqrt(tot);
+      *static_cast<CT*>(red.out) = static_cast<CT>(tot);
+    }
+    return;
+  }
   __shared__ bool last;
   if (threadIdx.x == 0) {
     pairs<CT>(red.part)[blockIdx.x] = make_pair_of<CT>(a.s, a.c);
@@ -964,8 +972,8 @@ FX_D void row_finish(const RowRed& rr, ThreadSum<CT> (&acc)[V], CT (&m)[V], int6
   if (!last) return;
   __threadfence();
   // the S partials of each of the thread's rows, in split order; for a
-  // fixed split a warp reads 32*V contiguous values; 8 splits in flight
-  constexpr int KU = 8;
+  // fixed split a warp reads 32*V contiguous values; KU splits in flight
+  constexpr int KU = 32 / V > 8 ? 32 / V : 8;
   if (ISMAX) {
     const CT* pm = static_cast<const CT*>(rr.partm);
     CT mm[V];
@@ -1194,7 +1202,7 @@ FX_D void bwd_bc_finish(const GradArgs& ga, int64_t r, int64_t R, int nvalid) {
       constexpr int b = bc_rank<LL, I>();
       T* dst = static_cast<T*>(ga.g[L::slot]);
       if (dst) {
-        constexpr int KU = 8;
+        constexpr int KU = 32 / V > 8 ? 32 / V : 8;
         const pair_t<CT>* part = pairs<CT>(ga.part) + int64_t(b) * ga.S * R + r;
         CompSum<CT> a[V];
 #pragma unroll

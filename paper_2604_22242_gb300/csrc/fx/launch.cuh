@@ -670,8 +670,9 @@ template <class E, bool ISMAX, int V>
 fx_status launch_row(const Run& r, const E& e, const Slots& sl, int64_t R, int64_t C, void* out) {
   using CT = ct_of<E>;
   using LL = leaves_t<E>;
-  // ~128 KB in flight per SM: 8 column vectors per thread for 1-2 leaves
-  constexpr int NT = 256, U = tl_size<LL>::value <= 2 ? 8 : 4, NS = 4;
+  // ~128 KB in flight per SM: 8 column vectors per thread for 1-2 leaves; 4
+  // in FP64, whose slow arithmetic wants more warps rather than more loads each
+  constexpr int NT = 256, U = !std::is_same<CT, double>::value && tl_size<LL>::value <= 2 ? 8 : 4, NS = 4;
   RowRed rr{};
   rr.out = out;
   auto space = [&](int64_t gx, int64_t S) -> fx_status {
