@@ -352,10 +352,19 @@ class Expr:
             pass
 
 
+def _current_stream_ptr():
+    """cudaStream_t of torch's current stream on the current device. Building
+    the torch.cuda.Stream object for it takes 3 us, half of a small call."""
+    torch = _torch()
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return int(torch.cuda.current_stream().cuda_stream)
+    return int(raw(torch.cuda.current_device()))
+
+
 def _stream_ptr(stream):
     if stream is None:
-        torch = _torch()
-        stream = torch.cuda.current_stream()
+        return _current_stream_ptr()
     return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
 
 
