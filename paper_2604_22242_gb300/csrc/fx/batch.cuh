@@ -24,6 +24,8 @@ struct BatchMat {
   const void* p[FX_MAX_SLOTS];
   int64_t ld[FX_MAX_SLOTS];
   int64_t rows, cols;
+  // k_batch_skew: the shift of column c is (csbase + c csld) mod W
+  uint32_t csbase, csld;
   int64_t first;   // first work item of this matrix
   int32_t ntiles;
   int32_t vec;     // every full vector of this matrix is aligned
@@ -36,6 +38,9 @@ struct BatchMat {
 struct BatchItem {
   int32_t mat;
   int32_t tile;
+};
+struct BatchTile {  // work item of k_batch_skew
+  int32_t mat, tr, tc, unused;
 };
 
 // ---------------------------------------------------------------- async tile pipeline
@@ -232,22 +237,13 @@ FX_D void load_tile_vec(Pack<LL, V, CT>& p, const char* buf, const BatchMat& m, 
 
 // Per-warp tile partials: FP32 pairs for FP32 trees (no FP64 conversion on
 // the hot kernel's slow FP64 pipe; the combine widens them), FP64 pairs for
-// FP64 trees. The partial buffer holds double2 slots either way.
+// FP64 trees (pair_t).
 FX_D void store_partial(double2* part, int64_t i, float s, float c) {
   reinterpret_cast<float2*>(part)[i] = make_float2(s, c);
 }
 FX_D void store_partial(double2* part, int64_t i, double s, double c) {
   part[i] = make_double2(s, c);
 }
-template <class RT> FX_D double2 load_partial(const double2* part, int64_t i) {
-  if constexpr (std::is_same<RT, double>::value) {
-    return __ldcg(part + i);
-  } else {
-    const float2 f = __ldcg(reinterpret_cast<const float2*>(part) + i);
-    return make_double2(double(f.x), double(f.y));
-  }
-}
-
 // VC: consecutive slots of one column a thread evaluates per step (its
 // vector width: 16 bytes of elements, or half that); copies and skews stay
 // in 16-byte chunks of W elements.
@@ -368,25 +364,132 @@ __global__ void __launch_bounds__(NT) k_batch_async(const E e, const BatchMat* _
   cpa::wait_pending<0>();
 }
 
-// One warp per matrix: its tiles' per-warp partials (nw per tile), in
-// order, summed in FP64.
-template <class RT>
-__global__ void __launch_bounds__(256) k_batch_combine(const BatchMat* __restrict__ mats,
-                                                       const int64_t nmat, const double2* part,
-                                                       const int sslot, const int nw) {
-  const int64_t i = int64_t(blockIdx.x) * 8 + threadIdx.x / 32;
-  const int lane = threadIdx.x % 32;
-  if (i >= nmat) return;  // whole warps leave together
-  const BatchMat& m = mats[i];
-  std::conditional_t<std::is_same<RT, double>::value, CompSum<double>, PlainSum<double>> a;
-  a.init();
-  for (int64_t k = lane; k < int64_t(m.ntiles) * nw; k += 32) {
-    const double2 q = load_partial<RT>(part, m.first * nw + k);
-    a.add(q.x);
-    a.add(q.y);
+// ---------------------------------------------------------------- skewed tiles
+//
+// k_batch_skew: the batch's tiles through skew_tile (skew.cuh): plain leaves
+// and Z as aligned 16-byte register vectors, transposed leaves as aligned
+// pieces staged in shared memory, two blocks of 512 threads per
+// SM (three of 256 for 2-byte types). The
+// cp.async kernel above copies transposed leaves element by element and has
+// room for one block per SM (4096 matrices FP32: 3526 us, against 2618 with
+// this one and the block-wide combine below); it stays for batches in which a matrix's plain
+// leaves and Z do not share their misalignment, and as launch-shape pipeline 1.
+//
+// Warp 0 reads the next item's descriptor, one 8-byte word per lane, while
+// the current tile loads, and the item after that, so that no tile waits for
+// a chain of dependent loads.
+template <int NIN> struct SkewMat {  // the words of BatchMat that a tile needs
+  const void* p[NIN + 1];
+  int64_t ld[NIN + 1];
+  int64_t rows, cols;
+  uint32_t csbase, csld;
+};
+struct MatSlots {
+  const void* const* p;
+  const int64_t* ld;
+  FX_D SlotView operator()(int slot) const { return SlotView{p[slot], ld[slot], 1}; }
+};
+// Word w of SkewMat in BatchMat's memory.
+template <int NIN> FX_D int skew_word(int w) {
+  constexpr int F = FX_MAX_SLOTS;
+  return w <= NIN ? w : (w < 2 * NIN + 2 ? F + w - NIN - 1 : 2 * F + w - 2 * NIN - 2);
+}
+template <int NIN> struct SkewNext {
+  uint64_t* word;
+  BatchTile* tile;
+  uint64_t w;
+  BatchTile t;
+  FX_D void operator()() const {
+    if (threadIdx.x < sizeof(SkewMat<NIN>) / 8) word[threadIdx.x] = w;
+    if (threadIdx.x == 0) *tile = t;
   }
-  warp_merge(a);
-  if (lane == 0) *static_cast<RT*>(const_cast<void*>(m.p[sslot])) = RT(a.s + a.c);
+};
+// Stores a tile's values and adds them to the thread's sum.
+template <class T, int KIND, class CT> struct SkewPut {
+  T* z;      // the tile's first element in Z
+  int ldz;
+  CT& sum;
+  template <class P, int V> FX_D void full(const P&, const CT (&v)[V], int rel, int cc) const {
+    if constexpr (KIND != FX_KIND_FULL_REDUCE) {
+      Raw<T, V> o;
+#pragma unroll
+      for (int j = 0; j < V; ++j) o.v[j] = narrow_to<T>::from(v[j]);
+      vstore(z + (rel + cc * ldz), o);
+    }
+    if constexpr (KIND != FX_KIND_ELEMENTWISE) {
+#pragma unroll
+      for (int j = 0; j < V; ++j) sum += v[j];
+    }
+  }
+  template <class P, int V>
+  FX_D void part(const P&, const CT (&v)[V], int rel, int cc, int lo, int hi) const {
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+      if (j < lo || j >= hi) continue;
+      if constexpr (KIND != FX_KIND_FULL_REDUCE) sstore(z + (rel + cc * ldz + j), narrow_to<T>::from(v[j]));
+      if constexpr (KIND != FX_KIND_ELEMENTWISE) sum += v[j];
+    }
+  }
+};
+
+template <class E, class T, int V, int TR, int TC, int NT, int KIND, int NIN>
+__global__ void __launch_bounds__(NT, skew_blocks(NT))
+    k_batch_skew(const E e, const BatchMat* __restrict__ mats, const BatchTile* __restrict__ tiles,
+                 const int64_t ntiles, double2* part) {
+  using SS = SkewShape<E, T, V, TR, TC, NT>;
+  using CT = typename SS::CT;
+  constexpr int NWORD = int(sizeof(SkewMat<NIN>) / 8);
+  static_assert(NWORD <= 32 && sizeof(SkewMat<NIN>) % 8 == 0, "one word per lane of warp 0");
+  __shared__ CT sm[SS::SMEM];
+  __shared__ uint64_t words[2][NWORD];
+  __shared__ BatchTile at[2];
+  const int64_t G = gridDim.x;
+  const int64_t last = ntiles - 1;
+  auto item = [&](int64_t i) { return tiles[i < ntiles ? i : last]; };
+  auto word = [&](const BatchTile& t) -> uint64_t {
+    const int w = int(threadIdx.x) < NWORD ? int(threadIdx.x) : 0;
+    return __ldg(reinterpret_cast<const unsigned long long*>(mats + t.mat) + skew_word<NIN>(w));
+  };
+  BatchTile next = {};
+  if (threadIdx.x < 32) {
+    const BatchTile t0 = item(blockIdx.x);
+    SkewNext<NIN>{words[0], &at[0], word(t0), t0}();
+    next = item(blockIdx.x + G);
+  }
+  __syncthreads();
+  int b = 0;
+  for (int64_t i = blockIdx.x; i < ntiles; i += G, b ^= 1) {
+    const SkewMat<NIN>& m = *reinterpret_cast<const SkewMat<NIN>*>(words[b]);
+    const BatchTile t = at[b];
+    SkewNext<NIN> fetched{words[b ^ 1], &at[b ^ 1], 0, next};
+    if (threadIdx.x < 32) {
+      fetched.w = word(next);
+      next = item(i + 2 * G);
+    }
+    CT tsum = CT(0);  // a thread adds at most TR * TC / NT values of a tile
+    const SkewPlace place{int(m.rows), int(m.cols), t.tr * TR, t.tc * TC, m.csbase, m.csld};
+    T* z = static_cast<T*>(const_cast<void*>(m.p[NIN])) + (place.r0 + place.c0 * m.ld[NIN]);
+    skew_tile<SS, T>(e, MatSlots{m.p, m.ld}, place, sm, fetched, SkewPut<T, KIND, CT>{z, int(m.ld[NIN]), tsum});
+    if constexpr (KIND != FX_KIND_ELEMENTWISE) {
+      ThreadSum<CT> st;
+      st.s = tsum;
+      st.c = CT(0);
+      warp_merge(st);
+      if ((threadIdx.x & 31) == 0)
+        store_partial(part, i * (NT / 32) + threadIdx.x / 32, st.s, st.c);
+    }
+  }
+}
+
+// One block per matrix: its tiles' per-warp partials (nw per tile) as pairs,
+// in a fixed order (block_sum_partials). A warp per matrix took 68 us for
+// 4096 matrices of up to 8192 partials, most of it waiting for one matrix.
+template <class RT>
+__global__ void __launch_bounds__(128) k_batch_combine(const BatchMat* __restrict__ mats,
+                                                       double2* part, const int sslot, const int nw) {
+  const BatchMat& m = mats[blockIdx.x];
+  const double tot = block_sum_partials<RT>(pairs<RT>(part) + m.first * nw, int64_t(m.ntiles) * nw);
+  if (threadIdx.x == 0) *static_cast<RT*>(const_cast<void*>(m.p[sslot])) = RT(tot);
 }
 
 struct BatchCacheEntry {
@@ -395,6 +498,8 @@ struct BatchCacheEntry {
   std::vector<fx_batch_item> items_seen;
   double scal_seen[FX_MAX_SCALARS] = {};
   bool built = false;
+  int pipe_seen = 0;      // launch-shape pipeline the work-list was built for
+  bool skewed = false;    // the work-list is of BatchTiles, for k_batch_skew
   int64_t n = 0, nitems = 0;
   Workspace dev;  // descriptors, items, partials
   BatchMat* mats = nullptr;
@@ -525,7 +630,8 @@ fx_status run_batch(fx_expr* x, const Root& root, int64_t n, const fx_batch_item
     if (!x->batch) x->batch = new (std::nothrow) BatchCache;
     if (!x->batch) return fail(FX_E_NOMEM, "out of host memory");
     BatchCacheEntry& c = x->batch->cur;
-    const bool same = c.built && c.mats && c.n == n &&
+    constexpr int STR = dbl ? 32 : 64, STC = 64;  // tiles of k_batch_skew
+    const bool same = c.built && c.mats && c.n == n && c.pipe_seen == x->tune.pipe &&
                       memcmp(c.scal_seen, x->scal, sizeof c.scal_seen) == 0 &&
                       (n == 0 || memcmp(c.items_seen.data(), items,
                                         size_t(n) * sizeof(fx_batch_item)) == 0);
@@ -543,6 +649,8 @@ fx_status run_batch(fx_expr* x, const Root& root, int64_t n, const fx_batch_item
       });
       std::vector<BatchMat> mats(n);
       std::vector<BatchItem> work;
+      std::vector<BatchTile> swork;
+      bool skewed = x->tune.pipe == 0 && V > 1 && V * sizeof(T) == 16 && tma_uniform<LL, T>();
       for (int64_t oi = 0; oi < n; ++oi) {
         const int64_t i = order[oi];
         const fx_batch_item& it = items[i];
@@ -595,36 +703,59 @@ fx_status run_batch(fx_expr* x, const Root& root, int64_t n, const fx_batch_item
           }
           m.skew = (ok && first >= 0) ? first + 1 : 0;
           m.sbase = m.skew ? int((reinterpret_cast<uintptr_t>(m.p[first]) / sizeof(T)) % W) : 0;
+          Binding lb[FX_MAX_SLOTS];
+          for (int k = 0; k < n_in; ++k) {
+            lb[k].p = const_cast<void*>(m.p[k]);
+            lb[k].ld = m.ld[k];
+          }
+          if (R > 0 && C > 0 &&
+              !skew_ok<LL, T, W>(lb, has_z ? m.p[zs] : nullptr, has_z ? m.ld[zs] : 0, m.csbase, m.csld))
+            skewed = false;
         }
-        // row tiles cover R plus the largest skew (W - 1 rows)
-        const int64_t nt = (R > 0 && C > 0)
-                               ? ((R + 16 / int64_t(sizeof(T)) - 1 + TR - 1) / TR) * ((C + TCc - 1) / TCc)
-                               : 0;
-        m.first = int64_t(work.size());
-        m.ntiles = int32_t(nt);
-        for (int64_t t = 0; t < nt; ++t) work.push_back(BatchItem{int32_t(i), int32_t(t)});
       }
+      for (int64_t oi = 0; oi < n; ++oi) {
+        const int64_t i = order[oi];
+        BatchMat& m = mats[i];
+        const int64_t R = m.rows, C = m.cols;
+        // row tiles cover R plus the largest shift
+        constexpr int W = 16 / int(sizeof(T));
+        const int64_t tr = skewed ? (R + max_shift<W>(m.csbase, m.csld, C) + STR - 1) / STR
+                                  : (R + W - 1 + TR - 1) / TR;
+        const int64_t tc = skewed ? (C + STC - 1) / STC : (C + TCc - 1) / TCc;
+        const int64_t nt = (R > 0 && C > 0) ? tr * tc : 0;
+        m.first = int64_t(skewed ? swork.size() : work.size());
+        m.ntiles = int32_t(nt);
+        for (int64_t t = 0; t < nt; ++t) {
+          if (skewed) swork.push_back(BatchTile{int32_t(i), int32_t(t % tr), int32_t(t / tr), 0});
+          else work.push_back(BatchItem{int32_t(i), int32_t(t)});
+        }
+      }
+      const size_t nwork = skewed ? swork.size() : work.size();
       if (c.exec) {
         cudaGraphExecDestroy(c.exec);
         c.exec = nullptr;
       }
       const size_t bm = ((sizeof(BatchMat) * n) + 255) & ~size_t(255);
-      const size_t bi = ((sizeof(BatchItem) * work.size()) + 255) & ~size_t(255);
-      const size_t bp = sizeof(double2) * (NTMAX / 32) * (work.size() > 0 ? work.size() : 1);
+      const size_t wb = skewed ? sizeof(BatchTile) * nwork : sizeof(BatchItem) * nwork;
+      const size_t bi = (wb + 255) & ~size_t(255);
+      const size_t bp = sizeof(double2) * (NTMAX / 32) * (nwork > 0 ? nwork : 1);
       FX_TRY(c.dev.ensure(bm + bi + bp, st));
       char* base = static_cast<char*>(c.dev.p);
       c.mats = reinterpret_cast<BatchMat*>(base);
       c.items = reinterpret_cast<BatchItem*>(base + bm);
       c.part = reinterpret_cast<double2*>(base + bm + bi);
       if (n > 0) FX_CUDA(cudaMemcpyAsync(c.mats, mats.data(), sizeof(BatchMat) * n, cudaMemcpyHostToDevice, st));
-      if (!work.empty())
-        FX_CUDA(cudaMemcpyAsync(c.items, work.data(), sizeof(BatchItem) * work.size(), cudaMemcpyHostToDevice, st));
+      if (nwork > 0)
+        FX_CUDA(cudaMemcpyAsync(c.items, skewed ? static_cast<const void*>(swork.data()) : work.data(), wb,
+                                cudaMemcpyHostToDevice, st));
       FX_CUDA(cudaStreamSynchronize(st));  // host vectors die at scope end
       c.items_seen.assign(items, items + n);
       memcpy(c.scal_seen, x->scal, sizeof c.scal_seen);
       c.built = true;
+      c.skewed = skewed;
+      c.pipe_seen = x->tune.pipe;
       c.n = n;
-      c.nitems = int64_t(work.size());
+      c.nitems = int64_t(nwork);
     }
     const E& e = inner_of(root);
     Run r = run_of(x, st);
@@ -660,9 +791,21 @@ fx_status run_batch(fx_expr* x, const Root& root, int64_t n, const fx_batch_item
     using B2 = std::integral_constant<int, 2>;
     using B3 = std::integral_constant<int, 3>;
     using B4 = std::integral_constant<int, 4>;
+    constexpr int SNT = skew_threads<T>();
+    auto launch_skew = [&]() -> fx_status {
+      if constexpr (V > 1 && V * sizeof(T) == 16 && tma_uniform<LL, T>()) {
+        constexpr int KE = kind == FX_KIND_MULTI ? FX_KIND_MULTI : KIND0;
+        auto kern = k_batch_skew<E, T, V, STR, STC, SNT, KE, NIN>;
+        const int grid = grid_for(kern, SNT, c.nitems, r.tune);
+        kern<<<grid, SNT, 0, st>>>(e, c.mats, reinterpret_cast<const BatchTile*>(c.items), c.nitems, c.part);
+      }
+      return after_launch(r, "k_batch_skew");
+    };
     auto launch_all = [&]() -> fx_status {
       if (c.nitems > 0) {
-        if (NTsel == 512) {
+        if (c.skewed) {
+          FX_TRY(launch_skew());
+        } else if (NTsel == 512) {
           if (NBsel == 2) FX_TRY(launch_one(I512{}, B2{}));
           else if (NBsel == 4) FX_TRY(launch_one(I512{}, B4{}));
           else FX_TRY(launch_one(I512{}, B3{}));
@@ -673,8 +816,8 @@ fx_status run_batch(fx_expr* x, const Root& root, int64_t n, const fx_batch_item
         }
       }
       if (has_s && c.n > 0) {
-        k_batch_combine<CT><<<unsigned((c.n + 7) / 8), 256, 0, st>>>(c.mats, c.n, c.part, sslot,
-                                                                     NTsel / 32);
+        k_batch_combine<CT><<<unsigned(c.n), 128, 0, st>>>(c.mats, c.part, sslot,
+                                                           (c.skewed ? SNT : NTsel) / 32);
         FX_TRY(after_launch(r, "k_batch_combine"));
       }
       return FX_OK;

@@ -12,6 +12,7 @@ pytestmark = pytest.mark.gpu
 # the last rows reached only by the shift (57 + 7 and 61 + 3 fill a tile)
 SHAPES = [(1, 1), (1, 70), (3, 2), (5, 67), (57, 65), (58, 64), (61, 63), (63, 7), (65, 130),
           (127, 9), (129, 128), (201, 71), (517, 203)]
+SHAPE = (256, 4, 1, 0)  # blocks_per_sm given: these tiles at any size
 
 
 @pytest.fixture(scope="module")
@@ -36,7 +37,7 @@ def test_skewed_tiles(fx, name, storage):
         pytest.skip("compiled for FP32")
     for k, (R, C) in enumerate(SHAPES):
         env = synth.operands(40 + k, specs_for(name, R, C), storage, "uniform")
-        check(name, storage, run(fx, name, storage, env, R, C), env, f" at {R}x{C}")
+        check(name, storage, run(fx, name, storage, env, R, C, shape=SHAPE), env, f" at {R}x{C}")
 
 
 @pytest.mark.parametrize("storage", ["f32", "f16"])
@@ -48,6 +49,6 @@ def test_residues_and_leading_dimensions(fx, storage):
         lds = {s: rows + pad + (w if s == "B" else 0) + (1 if s == "D" else 0)
                for s, rows, _ in specs_for(name, R, C)}
         env = synth.operands(60 + pad, specs_for(name, R, C), storage, "uniform", lds=lds)
-        check(name, storage, run(fx, name, storage, env, R, C, ldz=R + pad), env, f" pad {pad}")
+        check(name, storage, run(fx, name, storage, env, R, C, ldz=R + pad, shape=SHAPE), env, f" pad {pad}")
         # residues that differ: the general tile kernel
-        check(name, storage, run(fx, name, storage, env, R, C, ldz=R + pad + 1), env, f" pad {pad}, Z apart")
+        check(name, storage, run(fx, name, storage, env, R, C, ldz=R + pad + 1, shape=SHAPE), env, f" pad {pad}, Z apart")
