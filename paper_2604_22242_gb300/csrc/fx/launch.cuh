@@ -496,8 +496,21 @@ fx_status launch_tile_skew(const Run& r, const E& e, const Slots& sl, int64_t R,
   return FX_OK;
 }
 
+// Up to this many elements the register-staged tiles beat the TMA kernel,
+// which spends about a microsecond more on its barriers, descriptors and
+// output staging, and one block per SM on a matrix that the L2 cache serves
+// anyway. Z and s of 64^2 / 512^2 / 2048^2 FP32: 3.3 / 5.4 / 13.8 us against
+// 4.0 / 6.7 / 15.4, BF16 at 2048^2 11.4 against 11.6; at 3072^2 FP32 35.6
+// against 35.9, BF16 23.6 against 19.8. Transpose-closed trees, which read
+// each element once on the TMA kernel only: 512^2 3.0 against 4.2 us, 2048^2
+// 9.8 against 9.0.
+template <class LL> constexpr int64_t small_tiles() {
+  return flip_closed<LL>() ? int64_t(1) << 20 : int64_t(1) << 22;
+}
+
 // Tiles of a tree with transposed leaves. Launch-shape pipeline 0: the
-// TMA kernel when the operands allow it, else (unless aligned vectors do)
+// register tiles for small matrices (unless blocks_per_sm is given, which
+// asks for the TMA kernel), else the TMA kernel when the operands allow it, else (unless aligned vectors do)
 // the skewed tiles when the operands share their misalignment; 1: the cp.async pipeline when
 // every plain leaf and the output are vector-aligned; otherwise, and for
 // pipeline 2, the register-staged kernel.
@@ -506,6 +519,8 @@ fx_status launch_tiles(const Run& r, const E& e, const Slots& sl, int64_t R, int
                        const EpiV& ev, const Epi1& e1, RedArgs red) {
   using LL = leaves_t<E>;
   if constexpr (count_mt<LL>() > 0) {
+    if (r.tune.pipe == 0 && r.tune.bps == 0 && vec && R * C <= small_tiles<LL>())
+      return launch_tile<E, EpiV, V>(r, e, sl, R, C, ev, red);
     if (r.tune.pipe == 0) {
       bool used = false;
       const fx_status s = launch_tile_tma<T>(r, e, sl, R, C, ev, red, &used);
