@@ -123,11 +123,16 @@ FX_D int clamp_valid(int64_t left, int V) {
 
 // ---------------------------------------------------------------- leaf loads
 
+template <class T> struct bits_as { using type = T; };
+template <> struct bits_as<bf16> { using type = unsigned short; };
+template <> struct bits_as<f16> { using type = unsigned short; };
+
 // Flat layout: element i = r + c*R of every leaf. Matrix leaves are dense
-// (ld == R) and read at i; an each_col vector at r (i and R are multiples
-// of V, so the V elements share one column); an each_row vector at c.
+// (ld == R) and read at i; an each_col vector at r; an each_row vector at c
+// (only where V divides R, so that the V elements share one column). R is
+// passed only for trees with broadcast leaves.
 template <class LL, int V, class CT, int I = 0>
-FX_D void load_flat(Pack<LL, V, CT>& p, const Slots& sl, int64_t i, int64_t r, int64_t c) {
+FX_D void load_flat(Pack<LL, V, CT>& p, const Slots& sl, int64_t i, int64_t r, int64_t c, int64_t R) {
   if constexpr (I < tl_size<LL>::value) {
     using L = typename tl_at<LL, I>::type;
     using T = typename L::elem;
@@ -138,7 +143,16 @@ FX_D void load_flat(Pack<LL, V, CT>& p, const Slots& sl, int64_t i, int64_t r, i
     if constexpr (L::mode == MN) {
       vload(dst, base + i);
     } else if constexpr (L::mode == MBC) {
-      if (s.vs == 1) {
+      if (V > 1 && (uint32_t(R) & uint32_t(V - 1)) != 0) {
+        // the vector may run on into the next column's first rows; the
+        // vector leaf is read through L1, which holds it after one column
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+          const int64_t rj = r + j < R ? r + j : r + j - R;
+          *reinterpret_cast<typename bits_as<T>::type*>(&dst.v[j]) =
+              __ldg(reinterpret_cast<const typename bits_as<T>::type*>(base + rj * s.vs));
+        }
+      } else if (s.vs == 1) {
         vload(dst, base + r);
       } else {
 #pragma unroll
@@ -147,7 +161,7 @@ FX_D void load_flat(Pack<LL, V, CT>& p, const Slots& sl, int64_t i, int64_t r, i
     } else {
       dst.v[0] = sload(base + c * s.vs);
     }
-    load_flat<LL, V, CT, I + 1>(p, sl, i, r, c);
+    load_flat<LL, V, CT, I + 1>(p, sl, i, r, c, R);
   }
 }
 
@@ -559,7 +573,7 @@ template <class CT, bool SQRT, class S> FX_D void finish_full_reduce(S& a, const
 // ---------------------------------------------------------------- A3: flat stream
 
 // With broadcast leaves, (r, c) of element i comes from one division by R
-// per vector (FastDiv; the host guarantees n < 2^32 and R % V == 0).
+// per vector (FastDiv; the host guarantees n < 2^32 and R >= V).
 template <class E, class Epi, int V, int U>
 __global__ void __launch_bounds__(512) k_flat(const E e, const Slots sl, const int64_t n,
                                               const Epi epi, const RedArgs red, const FastDiv fd) {
@@ -590,7 +604,7 @@ __global__ void __launch_bounds__(512) k_flat(const E e, const Slots sl, const i
           c = fd.div(uint32_t(vi * V));
           r = vi * V - c * fd.d;
         }
-        load_flat(p[u], sl, vi * V, r, c);
+        load_flat(p[u], sl, vi * V, r, c, BC ? int64_t(fd.d) : 0);
       }
     }
     if constexpr (FMA64) {
@@ -631,10 +645,15 @@ __global__ void __launch_bounds__(512) k_flat(const E e, const Slots sl, const i
       }
     }
   }
-  if (V > 1 && !BC && blockIdx.x == 0) {  // the n % V trailing elements, one lane each
+  if (V > 1 && blockIdx.x == 0) {  // the n % V trailing elements, one lane each
     for (int64_t i = nv * V + threadIdx.x; i < n; i += bdim) {
       Pack<LL, 1, CT> q;
-      load_flat(q, sl, i, 0, 0);
+      int64_t r = 0, c = 0;
+      if constexpr (BC) {
+        c = fd.div(uint32_t(i));
+        r = i - c * fd.d;
+      }
+      load_flat(q, sl, i, r, c, BC ? int64_t(fd.d) : 0);
       CT v1[1];
       eval_lanes<1>(e, q, v1);
       CT v[V];
