@@ -391,7 +391,9 @@ fx_status run_umma32(fx_expr* x, const Root& root, cudaStream_t st, bool* used) 
   // Z written over an operand: the fallback for unsplittable values reads the
   // operands while other blocks store
   if (overlap(zb, a, sizeof(float)) || overlap(zb, b, sizeof(float))) return FX_OK;
-  const int64_t ntiles = ((M + u3::BM - 1) / u3::BM) * ((N + u3::BN - 1) / u3::BN);
+  const int sms = device_sms() > 0 ? device_sms() : 1;
+  const u3::Shape32 shape = u3::choose_shape(M, N, int((K + u3::BK - 1) / u3::BK), sms);
+  const int64_t ntiles = ((M + u3::BM - 1) / u3::BM) * ((N + shape.bn - 1) / shape.bn);
   const int64_t pieces = (int64_t(1) << 32) - 1;
   auto items = [](const Binding& o) { return (o.rows + 7) / 8 * o.cols; };
   if (ntiles >= (int64_t(1) << 26) || items(a) > pieces || items(b) > pieces) return FX_OK;
@@ -402,12 +404,11 @@ fx_status run_umma32(fx_expr* x, const Root& root, cudaStream_t st, bool* used) 
     cudaGetLastError();
     return FX_OK;
   }
-  const int sms = device_sms() > 0 ? device_sms() : 1;
-  const int S = u3::choose_splits(ntiles, int((K + u3::BK - 1) / u3::BK), sms);
+  const int S = shape.S;
   auto up = [](size_t v) { return (v + 255) & ~size_t(255); };
   auto ldp = [](const Binding& o) { return (o.rows + 7) / 8 * 8; };
   const size_t pa = up(size_t(ldp(a)) * size_t(a.cols) * 6), pb = up(size_t(ldp(b)) * size_t(b.cols) * 6);
-  const size_t pp = S > 1 ? size_t(ntiles) * S * u3::BM * u3::BN * sizeof(float) : 0;
+  const size_t pp = S > 1 ? size_t(ntiles) * S * u3::BM * shape.bn * sizeof(float) : 0;
   if (x->ws_gemm.ensure(pa + pb + pp, st) != FX_OK) {
     cudaGetLastError();
     return FX_OK;
@@ -428,16 +429,13 @@ fx_status run_umma32(fx_expr* x, const Root& root, cudaStream_t st, bool* used) 
     return true;
   };
   if (!planes(a, da, AMN ? 64 : u3::BM, {u3::A1, u3::A2, u3::A3}) ||
-      !planes(b, db, BMN ? 64 : u3::BN, {u3::B1, u3::B2, u3::B3}))
+      !planes(b, db, BMN ? 64 : shape.bn, {u3::B1, u3::B2, u3::B3}))
     return FX_OK;
   auto split = [&](const Binding& o, bf16* d) {
     return u3::SplitArgs{static_cast<const float*>(o.p), d, o.rows, o.cols, o.ld, ldp(o), items(o),
                          FastDiv::make(uint32_t((o.rows + 7) / 8)),
                          aligned(o.p, 16) && o.ld % 4 == 0 ? 1 : 0};
   };
-  auto kern = u3::k_gemm_umma32<AMN, BMN, Lifted, PS>;
-  const int smem = 2 * u3::NP * u3::TILE + 1024 + int(sizeof(u3::Bars));
-  FX_TRY(allow_smem(kern, smem));
   *used = true;
   x->last_launches = 0;
   const int64_t blocks = (items(a) + items(b) + 255) / 256;
@@ -448,10 +446,19 @@ fx_status run_umma32(fx_expr* x, const Root& root, cudaStream_t st, bool* used) 
   const int64_t nitems = ntiles * S;
   const u3::Source sa{static_cast<const float*>(a.p), AMN ? 1 : a.ld, AMN ? a.ld : 1};
   const u3::Source sb{static_cast<const float*>(b.p), BMN ? 1 : b.ld, BMN ? b.ld : 1};
-  kern<<<unsigned(nitems < sms ? nitems : sms), u3::THREADS, smem, st>>>(
-      maps, LR::make(root), make_slots(x->b, NIN), static_cast<float*>(zb.p), zb.ld, int(M), int(N),
-      int(K), S, part, tick + 2, tick, sa, sb, err);
-  return after_launch(r, "k_gemm_umma32");
+  auto launch = [&](auto bn) -> fx_status {
+    constexpr int BN = decltype(bn)::value;
+    using SL = u3::Slots32<BN>;
+    auto kern = u3::k_gemm_umma32<BN, AMN, BMN, Lifted, PS>;
+    const int smem = int(SL::bytes) + 1024 + int(sizeof(u3::Bars));
+    FX_TRY(allow_smem(kern, smem));
+    kern<<<unsigned(nitems < sms ? nitems : sms), SL::THREADS, smem, st>>>(
+        maps, LR::make(root), make_slots(x->b, NIN), static_cast<float*>(zb.p), zb.ld, int(M), int(N),
+        int(K), S, part, tick + 2, tick, sa, sb, err);
+    return after_launch(r, "k_gemm_umma32");
+  };
+  if (shape.bn == 256) return launch(std::integral_constant<int, 256>{});
+  return launch(std::integral_constant<int, 128>{});
 }
 
 // A tree with matrix products: products into temporaries (slots NIN ..

@@ -10,25 +10,26 @@
 // the product.
 //
 // Accumulation. The tensor cores' FP32 accumulator cuts instead of rounding
-// and a long sum in it drifts, so no sum of leading products (a1 b1) is
-// longer than one K block of 64 there: the epilogue warps read it out and
-// add it to their registers with rounded FP32 adds. The five small products,
-// at most 2^-8 of the leading one, keep one accumulator for the whole tile.
+// and a long sum in it drifts, so no sum is longer than one K block of 64
+// there: the five small products first (at most 2^-8 of the leading one, so
+// their twenty cuts are small), then a1 b1; the epilogue warps read the block
+// out and add it to their registers with rounded FP32 adds. Two accumulators
+// alternate by block.
 //
-// Layout: 128 x 128 tiles, K blocks of 64. A block is six 16 KB plane tiles
-// (a3 b1 a1 b3 a2 b2, in the order of their first use); two blocks are in
-// shared memory, every plane tile with its own full / empty mbarriers, so a
-// plane's slot refills as soon as its last product has read it. Per SM and
-// block: 96 KB from L2 for 24 tcgen05.mma of 128 x 128 x 16, 64 bytes per
-// clock at the tensor cores' rate (a BF16 product with 128 x 256 tiles needs
-// 96). TMEM (512 columns): two leading accumulators, alternating by K block,
-// and two small-product accumulators, alternating by tile.
+// Layout: 128 x BN tiles (BN 256, or 128 where that leaves SMs idle), K
+// blocks of 64. One thread issues all products, so their number counts:
+// 24 tcgen05.mma a block, 128 clocks each at N = 256 but 64 at N = 128, which
+// is also bound by shared memory (operand reads and TMA writes, 187 bytes per
+// clock against 141 at N = 256). Descriptors are a constant plus an address.
+// Every plane tile of a block has its own full / empty mbarriers, and the
+// products are ordered so that a plane's slot is free as early as possible:
+// with N = 256, a1, b1, a2 and a3 have two slots, b2 and b3 one (224 KB); with
+// N = 128 all have two (192 KB).
 //
 //   warp 0      lane 0 issues the TMA loads
 //   warp 1      owns the TMEM; lane 0 issues the products
-//   warps 2-9   the epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31, the
-//               first four warps columns 0-63 of the tile, the others 64-127
-//               (64 sums a thread; 128 would spill at ten warps). While they
+//   others      the epilogue, BN / 16 warps: warp w reads TMEM lanes
+//               32 (w % 4) .. + 31 and 64 columns (64 sums a thread). While they
 //               store a tile, the next one's first two K blocks are multiplied.
 //
 // A work item is a tile and one of S contiguous ranges of its K blocks. With
@@ -36,8 +37,9 @@
 // items to finish (a ticket; no block waits for another) adds the S partials
 // in range order and evaluates the remainder.
 //
-// Measured with sigmoid(s X Y + W) at 2048 x 1536 x 2048: 107 us, against
-// 268 us for the library's FP32 GEMM and the element-wise pass after it; the
+// Measured with sigmoid(s X Y + W) at 2048 x 1536 x 2048: 94 us (107 with
+// 128-column tiles only and descriptors computed per product), against 268 us
+// for the library's FP32 GEMM and the element-wise pass after it; the
 // product's error against 64 bits is smaller (maximum of the result 8.7e-8
 // against 1.0e-7 at K = 2048, 9.0e-8 against 1.6e-7 at K = 700).
 //
@@ -56,13 +58,38 @@ namespace umma32 {
 using umma::fence_after;
 using umma::fence_before;
 
-constexpr int BM = 128, BN = 128, BK = 64, UK = 16;
-constexpr int TILE = BM * BK * 2;  // one plane tile of either operand
-constexpr int NP = 6;              // plane tiles of a K block
-constexpr int EPI_WARPS = 8;
-constexpr int NC = BN / 2;         // columns an epilogue thread sums
-constexpr int THREADS = 64 + 32 * EPI_WARPS;
-enum Plane : int { A3 = 0, B1 = 1, A1 = 2, B3 = 3, A2 = 4, B2 = 5 };
+constexpr int BM = 128, BK = 64, UK = 16;
+constexpr int UNIT = 128 * BK * 2;  // shared memory of 128 rows of a plane's block
+constexpr int NP = 6;               // plane tiles of a K block
+constexpr int NC = 64;              // columns an epilogue thread sums
+enum Plane : int { A1 = 0, A2 = 1, A3 = 2, B1 = 3, B2 = 4, B3 = 5 };
+
+// Slots of the planes for tiles of BN columns. Plane p of K block g is in slot
+// g % depth(p); its barriers are bar(p, g), its memory at at(p, g), and it is
+// the use(p, g)-th block there.
+template <int BN> struct Slots32 {
+  static constexpr int units(int p) { return p >= B1 ? BN / 128 : 1; }
+  FX_HD static constexpr uint32_t depth(int p) { return BN == 256 && (p == B2 || p == B3) ? 1 : 2; }
+  FX_HD static constexpr uint32_t base(int p) {
+    uint32_t u = 0;
+    for (int q = 0; q < p; ++q) u += depth(q) * uint32_t(q >= B1 ? BN / 128 : 1);
+    return u * uint32_t(UNIT);
+  }
+  FX_HD static constexpr uint32_t pick(int p, uint32_t g) { return depth(p) == 2 ? g & 1u : 0u; }
+  FX_HD static constexpr uint32_t use(int p, uint32_t g) { return depth(p) == 2 ? g >> 1 : g; }
+  FX_HD static constexpr uint32_t bar(int p, uint32_t g) { return uint32_t(p) * 2u + pick(p, g); }
+  FX_HD static constexpr uint32_t at(int p, uint32_t g) {
+    return base(p) + pick(p, g) * uint32_t(UNIT) * uint32_t(p >= B1 ? BN / 128 : 1);
+  }
+  static constexpr uint32_t bytes = base(NP);
+  static constexpr int EPI_WARPS = BN / 16, THREADS = 64 + 32 * EPI_WARPS;
+  // The order in which the producer loads a block's planes: a plane whose
+  // slot frees late does not hold up one that is free.
+  FX_HD static constexpr int order(int i) {
+    constexpr int o256[NP] = {A3, A1, B1, A2, B3, B2}, o128[NP] = {A3, B3, A2, B2, A1, B1};
+    return BN == 256 ? o256[i] : o128[i];
+  }
+};
 
 struct Maps {
   CUtensorMap m[NP];  // indexed by Plane
@@ -74,13 +101,12 @@ struct Source {
   int64_t s_mn, s_k;
 };
 struct Bars {
-  uint64_t full[2][NP], empty[2][NP];
-  uint64_t hif[2], hie[2];  // leading accumulator complete / read out (one arrival per warp)
-  uint64_t loe[2];          // small-product accumulator read out (one arrival per warp)
+  uint64_t full[2 * NP], empty[2 * NP];
+  uint64_t accf[2], acce[2];  // accumulator complete / read out (one arrival per warp)
   uint64_t drain;
   uint32_t taddr;
   volatile int abort;
-  int last;                 // this item completes its tile
+  int last;                   // this item completes its tile
 };
 
 // ---------------------------------------------------------------- planes
@@ -149,47 +175,36 @@ static __global__ void __launch_bounds__(256) k_split3(const SplitArgs a, const 
 
 // ---------------------------------------------------------------- product
 
-FX_D void ld32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
-      "%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]),
-        "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-        "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-}
-
-template <bool AMN, bool BMN> FX_HD constexpr uint32_t idesc() {  // kind::f16, BF16 in, FP32 out
+template <int BN, bool AMN, bool BMN> FX_HD constexpr uint32_t idesc() {  // BF16 in, FP32 out
   return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(AMN) << 15) | (uint32_t(BMN) << 16) |
          (uint32_t(BN >> 3) << 17) | (uint32_t(BM >> 4) << 24);
 }
 
-// One plane tile: rows mn0 .. mn0 + 127 of the operand, K block k0.
-template <bool MNMAJOR>
+// One plane tile: rows mn0 .. mn0 + ROWS - 1 of the operand, K block k0.
+template <bool MNMAJOR, int ROWS>
 FX_D void load_plane(char* dst, const CUtensorMap* m, int mn0, int k0, uint64_t* bar) {
-  tma::arrive_expect_tx(bar, TILE);
+  tma::arrive_expect_tx(bar, uint32_t(ROWS * BK * 2));
   if (MNMAJOR) {
-    tma::load_2d(dst, m, mn0, k0, bar);
-    tma::load_2d(dst + TILE / 2, m, mn0 + 64, k0, bar);
+#pragma unroll
+    for (int j = 0; j < ROWS / 64; ++j) tma::load_2d(dst + j * (UNIT / 2), m, mn0 + 64 * j, k0, bar);
   } else {
     tma::load_2d(dst, m, k0, mn0, bar);
   }
 }
-template <bool MNMAJOR> FX_D uint64_t plane_desc(uint32_t s, int k) {
-  return MNMAJOR ? umma::desc(s + uint32_t(k) * UK * 128, TILE / 2, 1024)
-                 : umma::desc(s + uint32_t(k) * UK * 2, 16, 1024);
+// The matrix descriptor of a plane tile at shared address 0, and its step per
+// 16 of K, in the descriptor's 16-byte units.
+template <bool MNMAJOR> FX_D uint64_t plane_desc() {
+  return umma::desc(0, MNMAJOR ? UNIT / 2 : 16, 1024);
 }
+template <bool MNMAJOR> FX_HD constexpr uint32_t kstep() { return (MNMAJOR ? UK * 128 : UK * 2) / 16; }
 
 // A thread's row m of Z, columns n0 .. n0 + NC - 1, from the product values acc;
-// the other leaves' values are loaded one piece of 16 columns ahead.
+// the other leaves' values are loaded one piece of 8 columns ahead.
 template <class T, class E, int PS>
 FX_D void store_row(const E& e, const Slots& sl, float* z, int64_t ldz, int64_t m, int n0, int N,
                     const float (&acc)[NC]) {
   using LL = leaves_t<E>;
-  constexpr int NL = tl_size<LL>::value, CW = 16;
+  constexpr int NL = tl_size<LL>::value, CW = 8;
   T wn[NL][CW], wc[NL][CW];
   if (n0 < N) umma::load_others<LL, PS, T, CW>(wn, sl, m, n0, N - n0 < CW ? N - n0 : CW);
 #pragma unroll
@@ -215,9 +230,26 @@ FX_D void store_row(const E& e, const Slots& sl, float* z, int64_t ldz, int64_t 
   }
 }
 
+// Brings the other leaves' part of a tile towards L2 while it is multiplied:
+// thread i of the epilogue takes half a column (256 bytes).
+template <class LL, int PS, int I = 0>
+FX_D void prefetch_others(const Slots& sl, int64_t m, int64_t n, int M) {
+  if constexpr (I < tl_size<LL>::value) {
+    using L = typename tl_at<LL, I>::type;
+    if constexpr (L::slot != PS) {
+      const SlotView& s = sl.s[L::slot];
+      const float* p = static_cast<const float*>(s.p) + m + n * s.ld;
+#pragma unroll
+      for (int j = 0; j < 64; j += 32)
+        if (m + j < M) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + j));
+    }
+    prefetch_others<LL, PS, I + 1>(sl, m, n, M);
+  }
+}
+
 // The product by FP32 fma from the operands themselves (unsplittable values):
 // 256 threads, 8 x 8 results each, K steps of 16 through shared memory.
-template <class E, int PS>
+template <int BN, class E, int PS>
 FX_D void fma_tiles(char* smem, const E& e, const Slots& sl, float* z, int64_t ldz, int M, int N,
                     int K, const Source& A, const Source& B, int tiles_m, int tiles_n) {
   using LL = leaves_t<E>;
@@ -225,10 +257,11 @@ FX_D void fma_tiles(char* smem, const E& e, const Slots& sl, float* z, int64_t l
   float* sa = reinterpret_cast<float*>(smem);
   float* sb = sa + KS * LDS;
   const int tid = threadIdx.x, tx = tid % 16, ty = (tid / 16) % 16;
-  for (int t = blockIdx.x; t < tiles_m * tiles_n; t += gridDim.x) {
+  constexpr int HALVES = BN / 128;  // 128 columns at a time
+  for (int th = blockIdx.x; th < tiles_m * tiles_n * HALVES; th += gridDim.x) {
     int tm, tn;
-    umma::tile_of(t, tiles_m, tiles_n, tm, tn);
-    const int m0 = tm * BM, n0 = tn * BN;
+    umma::tile_of(th / HALVES, tiles_m, tiles_n, tm, tn);
+    const int m0 = tm * BM, n0 = tn * BN + th % HALVES * 128;
     float acc[8][8];
 #pragma unroll
     for (int i = 0; i < 8; ++i)
@@ -282,16 +315,17 @@ FX_D void fma_tiles(char* smem, const E& e, const Slots& sl, float* z, int64_t l
   }
 }
 
-template <bool AMN, bool BMN, class E, int PS>
-__global__ void __launch_bounds__(THREADS, 1)
+template <int BN, bool AMN, bool BMN, class E, int PS>
+__global__ void __launch_bounds__(Slots32<BN>::THREADS, 1)
     k_gemm_umma32(const __grid_constant__ Maps maps, const E e, const Slots sl, float* z,
                   const int64_t ldz, const int M, const int N, const int K, const int S,
                   float* part, unsigned int* tickets, unsigned int* flag, const Source srcA,
                   const Source srcB, unsigned int* err) {
+  using SL = Slots32<BN>;
   extern __shared__ char smem_raw[];
   char* smem = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                        ~uintptr_t(1023));
-  Bars& bars = *reinterpret_cast<Bars*>(smem + 2 * NP * TILE);
+  Bars& bars = *reinterpret_cast<Bars*>(smem + SL::bytes);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int tiles_m = (M + BM - 1) / BM, tiles_n = (N + BN - 1) / BN;
   const int ntiles = tiles_m * tiles_n;
@@ -305,36 +339,36 @@ __global__ void __launch_bounds__(THREADS, 1)
     flag[1] = 0u;
   }
   if (direct) {
-    fma_tiles<E, PS>(smem, e, sl, z, ldz, M, N, K, srcA, srcB, tiles_m, tiles_n);
+    fma_tiles<BN, E, PS>(smem, e, sl, z, ldz, M, N, K, srcA, srcB, tiles_m, tiles_n);
     return;
   }
   if (threadIdx.x == 0) {
+    for (int i = 0; i < 2 * NP; ++i) {
+      tma::mbar_init(&bars.full[i], 1);
+      tma::mbar_init(&bars.empty[i], 1);
+    }
     for (int b = 0; b < 2; ++b) {
-      for (int p = 0; p < NP; ++p) {
-        tma::mbar_init(&bars.full[b][p], 1);
-        tma::mbar_init(&bars.empty[b][p], 1);
-      }
-      tma::mbar_init(&bars.hif[b], 1);
-      tma::mbar_init(&bars.hie[b], EPI_WARPS);
-      tma::mbar_init(&bars.loe[b], EPI_WARPS);
+      tma::mbar_init(&bars.accf[b], 1);
+      tma::mbar_init(&bars.acce[b], SL::EPI_WARPS);
     }
     tma::mbar_init(&bars.drain, 1);
     bars.abort = 0;
     tma::fence_mbar_init();
   }
   if (warp == 1) {
-    umma::tmem_alloc(&bars.taddr, 512);
+    umma::tmem_alloc(&bars.taddr, 2 * BN);
     umma::tmem_relinquish();
   }
   fence_before();
   __syncthreads();
   fence_after();
   const uint32_t tbase = bars.taddr;
-  // leading accumulators at columns 0 and 128, small-product ones at 256 and 384
 
   if (warp == 0) {
     if (lane == 0) {
-      uint32_t g = 0;  // K blocks so far
+      uint32_t g = 0;   // K blocks so far
+      uint32_t gf = 0;  // where the producer gave up: block and position in the order
+      int pf = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
         const int s = it / ntiles;
@@ -343,95 +377,91 @@ __global__ void __launch_bounds__(THREADS, 1)
         const int m0 = tm * BM, n0 = tn * BN;
         const int kb1 = int(int64_t(nk) * (s + 1) / S);
         for (int kb = int(int64_t(nk) * s / S); kb < kb1 && ok; ++kb, ++g) {
-          const int b = int(g & 1u);
-          char* st = smem + b * NP * TILE;
           const int k0 = kb * BK;
-          int p = 0;
-          for (; p < NP; ++p) {
-            if (g >= 2 && !tma::wait(&bars.empty[b][p], ((g >> 1) - 1u) & 1u, err)) {
+#pragma unroll
+          for (int o = 0; o < NP; ++o) {
+            const int p = SL::order(o);
+            const uint32_t i = SL::bar(p, g), use = SL::use(p, g);
+            if (ok && use >= 1 && !tma::wait(&bars.empty[i], (use - 1u) & 1u, err)) {
               ok = false;
-              break;
+              gf = g;
+              pf = o;
             }
-            if (p == B1 || p == B2 || p == B3)
-              load_plane<BMN>(st + p * TILE, &maps.m[p], n0, k0, &bars.full[b][p]);
-            else
-              load_plane<AMN>(st + p * TILE, &maps.m[p], m0, k0, &bars.full[b][p]);
+            if (!ok) continue;
+            if (p >= B1) load_plane<BMN, BN>(smem + SL::at(p, g), &maps.m[p], n0, k0, &bars.full[i]);
+            else load_plane<AMN, BM>(smem + SL::at(p, g), &maps.m[p], m0, k0, &bars.full[i]);
           }
-          if (!ok) {  // wait (bounded) for what is still in flight (here g >= 2)
-            bars.abort = 1;
-            for (int j = 0; j < NP; ++j) {
-              tma::wait(&bars.full[b ^ 1][j], ((g - 1u) >> 1) & 1u, nullptr);
-              tma::wait(&bars.full[b][j], ((g >> 1) - (j < p ? 0u : 1u)) & 1u, nullptr);
-            }
-          }
+        }
+      }
+      if (!ok) {  // wait (bounded) for the copies still in flight
+        bars.abort = 1;
+        for (int o = 0; o < NP; ++o) {
+          const int p = SL::order(o);
+          const uint32_t n = gf + (o < pf ? 1u : 0u);  // blocks whose plane p was issued
+          for (uint32_t j = n > SL::depth(p) ? n - SL::depth(p) : 0u; j < n; ++j)
+            tma::wait(&bars.full[SL::bar(p, j)], SL::use(p, j) & 1u, nullptr);
         }
       }
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      constexpr uint32_t ID = idesc<AMN, BMN>();
+      constexpr uint32_t ID = idesc<BN, AMN, BMN>();
+      const uint64_t da = plane_desc<AMN>(), db = plane_desc<BMN>();
+      const uint32_t s16 = tma::saddr(smem) >> 4;
       uint32_t g = 0;
-      int i = 0;  // items so far
       bool ok = true;
-      for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x, ++i) {
+      for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
         const int s = it / ntiles;
-        const int kb0 = int(int64_t(nk) * s / S), kb1 = int(int64_t(nk) * (s + 1) / S);
-        if (i >= 2 && !tma::wait(&bars.loe[i & 1], uint32_t((i - 2) >> 1) & 1u, err)) {
-          ok = false;
-          break;
-        }
-        const uint32_t lo = tbase + 256u + uint32_t(i & 1) * BN;
-        for (int kb = kb0; kb < kb1 && ok; ++kb, ++g) {
-          const int b = int(g & 1u);
-          const uint32_t par = (g >> 1) & 1u;
-          const uint32_t st = tma::saddr(smem + b * NP * TILE);
-          const uint32_t hi = tbase + uint32_t(b) * BN;
+        const int nkb = int(int64_t(nk) * (s + 1) / S) - int(int64_t(nk) * s / S);
+        for (int kb = 0; kb < nkb && ok; ++kb, ++g) {
+          const uint32_t acc = tbase + (g & 1u) * BN;
           auto ready = [&](int p) {
-            if (ok && !tma::wait(&bars.full[b][p], par, err)) ok = false;
+            if (ok && !tma::wait(&bars.full[SL::bar(p, g)], SL::use(p, g) & 1u, err)) ok = false;
           };
-          auto product = [&](int pa, int pb, uint32_t d, bool fresh) {
+          auto release = [&](int p) { umma::commit(&bars.empty[SL::bar(p, g)]); };
+          auto product = [&](int pa, int pb, bool fresh) {
+            const uint64_t a = da | uint64_t(s16 + (SL::at(pa, g) >> 4));
+            const uint64_t b = db | uint64_t(s16 + (SL::at(pb, g) >> 4));
 #pragma unroll
             for (int k = 0; k < BK / UK; ++k)
-              umma::mma(d, plane_desc<AMN>(st + uint32_t(pa * TILE), k),
-                        plane_desc<BMN>(st + uint32_t(pb * TILE), k), ID, (!fresh || k > 0) ? 1u : 0u);
+              umma::mma(acc, a + uint32_t(k) * kstep<AMN>(), b + uint32_t(k) * kstep<BMN>(), ID,
+                        (!fresh || k > 0) ? 1u : 0u);
           };
+          // the epilogue has read out the block this accumulator held before
+          if (g >= 2 && !tma::wait(&bars.acce[g & 1u], ((g >> 1) - 1u) & 1u, err)) ok = false;
           ready(A3);
           ready(B1);
           if (!ok) break;
           fence_after();
-          product(A3, B1, lo, kb == kb0);
-          umma::commit(&bars.empty[b][A3]);
+          product(A3, B1, true);
+          release(A3);
           ready(A1);
           ready(B3);
           if (!ok) break;
           fence_after();
-          product(A1, B3, lo, false);
-          umma::commit(&bars.empty[b][B3]);
+          product(A1, B3, false);
+          release(B3);
           ready(A2);
+          if (!ok) break;
+          fence_after();
+          product(A2, B1, false);
           ready(B2);
           if (!ok) break;
           fence_after();
-          product(A2, B2, lo, false);
-          product(A2, B1, lo, false);
-          umma::commit(&bars.empty[b][A2]);
-          product(A1, B2, lo, false);
-          umma::commit(&bars.empty[b][B2]);
-          // the epilogue has read out the block this accumulator held before
-          if (g >= 2 && !tma::wait(&bars.hie[b], ((g >> 1) - 1u) & 1u, err)) {
-            ok = false;
-            break;
-          }
-          fence_after();
-          product(A1, B1, hi, true);
-          umma::commit(&bars.empty[b][A1]);
-          umma::commit(&bars.empty[b][B1]);
-          umma::commit(&bars.hif[b]);
+          product(A1, B2, false);
+          product(A2, B2, false);
+          release(A2);
+          release(B2);
+          product(A1, B1, false);
+          release(A1);
+          release(B1);
+          umma::commit(&bars.accf[g & 1u]);
         }
       }
       if (!ok) {  // wake the epilogue (it sees the abort) after what was issued
         bars.abort = 1;
-        umma::commit(&bars.hif[0]);
-        umma::commit(&bars.hif[1]);
+        umma::commit(&bars.accf[0]);
+        umma::commit(&bars.accf[1]);
       }
       umma::commit(&bars.drain);
       tma::wait(&bars.drain, 0u, err);
@@ -443,47 +473,47 @@ __global__ void __launch_bounds__(THREADS, 1)
     const uint32_t tmine = tbase + (uint32_t(q * 32) << 16) + uint32_t(col);
     const int row = q * 32 + lane;
     uint32_t g = 0;
-    int i = 0;
-    for (int it = blockIdx.x; it < nitems; it += gridDim.x, ++i) {
+    for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
       const int s = it / ntiles, t = it - s * ntiles;
       const int nkb = int(int64_t(nk) * (s + 1) / S) - int(int64_t(nk) * s / S);
       bool ready = true;
+      int tm, tn;
+      umma::tile_of(t, tiles_m, tiles_n, tm, tn);
+      if (s == S - 1) {
+        const int i = int(threadIdx.x) - 64, n = tn * BN + i / 2;
+        if (n < N) prefetch_others<leaves_t<E>, PS>(sl, int64_t(tm) * BM + (i & 1) * 64, n, M);
+      }
       float acc[NC];
 #pragma unroll
       for (int j = 0; j < NC; ++j) acc[j] = 0.0f;
-      auto add_tmem = [&](uint32_t at) {
-#pragma unroll
-        for (int c = 0; c < NC / 32; ++c) {
-          uint32_t r[32];
-          ld32(at + uint32_t(c * 32), r);
-          umma::wait_ld();
-#pragma unroll
-          for (int j = 0; j < 32; ++j) acc[c * 32 + j] += __uint_as_float(r[j]);
-        }
-        fence_before();
-        __syncwarp();
-      };
       for (int kb = 0; kb < nkb; ++kb, ++g) {
-        const int b = int(g & 1u);
-        ready = tma::wait(&bars.hif[b], (g >> 1) & 1u, err);
+        const uint32_t b = g & 1u;
+        ready = tma::wait(&bars.accf[b], (g >> 1) & 1u, err);
         fence_after();
         // the TMEM loads are warp-wide: the warp decides together
         ready = __all_sync(0xffffffffu, ready && !bars.abort);
         if (!ready) break;
-        add_tmem(tmine + uint32_t(b) * BN);
-        if (lane == 0) tma::arrive(&bars.hie[b]);
+#pragma unroll
+        for (int c = 0; c < NC / 16; ++c) {
+          uint32_t r[16];
+          umma::ld16(tmine + b * BN + uint32_t(c * 16), r);
+          umma::wait_ld();
+#pragma unroll
+          for (int j = 0; j < 16; ++j) acc[c * 16 + j] += __uint_as_float(r[j]);
+        }
+        fence_before();
+        __syncwarp();
+        if (lane == 0) tma::arrive(&bars.acce[b]);
       }
       if (!ready) break;
-      add_tmem(tmine + 256u + uint32_t(i & 1) * BN);
-      if (lane == 0) tma::arrive(&bars.loe[i & 1]);
       if (S > 1) {
         float* mine = part + int64_t(it) * (BM * BN) + col * BM + row;
 #pragma unroll
         for (int j = 0; j < NC; ++j) __stcg(mine + j * BM, acc[j]);
         __threadfence();
-        asm volatile("bar.sync 1, %0;" ::"n"(32 * EPI_WARPS) : "memory");
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * SL::EPI_WARPS) : "memory");
         if (warp == 2 && lane == 0) bars.last = atomicAdd(tickets + t, 1u) == unsigned(S - 1);
-        asm volatile("bar.sync 1, %0;" ::"n"(32 * EPI_WARPS) : "memory");
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * SL::EPI_WARPS) : "memory");
         if (!bars.last) continue;
         __threadfence();
         if (warp == 2 && lane == 0) tickets[t] = 0u;  // ready for the next launch
@@ -495,8 +525,6 @@ __global__ void __launch_bounds__(THREADS, 1)
           for (int j = 0; j < NC; ++j) acc[j] += __ldcg(p + j * BM);
         }
       }
-      int tm, tn;
-      umma::tile_of(t, tiles_m, tiles_n, tm, tn);
       const int64_t m = int64_t(tm) * BM + row;
       if (m < M) store_row<float, E, PS>(e, sl, z, ldz, m, tn * BN + col, N, acc);
     }
@@ -505,23 +533,32 @@ __global__ void __launch_bounds__(THREADS, 1)
   __syncthreads();
   if (warp == 1) {
     fence_after();
-    umma::tmem_dealloc(tbase, 512);
+    umma::tmem_dealloc(tbase, 2 * BN);
   }
 }
 
-// K ranges per tile: the S that minimises waves of work items times their
-// length. In K blocks of 64 (about 0.8 us each): an item costs its own blocks
-// and about two to fill and drain its pipeline, one more to write and add
-// partials when S > 1.
-inline int choose_splits(int64_t ntiles, int nk, int sms) {
-  int best = 1;
-  int64_t cost = 0;
-  for (int S = 1; S <= 16 && S <= nk; ++S) {
-    const int64_t waves = (ntiles * S + sms - 1) / sms;
-    const int64_t c = waves * ((nk + S - 1) / S + 2 + (S > 1 ? 1 : 0));
-    if (S == 1 || c < cost) {
-      cost = c;
-      best = S;
+// Tile width and K ranges per tile: the pair that minimises waves of work
+// items times their length, in K blocks of a 128-column tile. An item costs
+// its own blocks (two units each at 256 columns) and about two to fill and
+// drain its pipeline, and with S > 1 one more to write its partial tile, per
+// 128 columns, and S to add them up.
+struct Shape32 {
+  int bn, S;
+};
+inline Shape32 choose_shape(int64_t M, int64_t N, int nk, int sms) {
+  Shape32 best{256, 1};
+  int64_t cost = -1;
+  for (int bn : {256, 128}) {
+    const int64_t ntiles = ((M + BM - 1) / BM) * ((N + bn - 1) / bn);
+    for (int S = 1; S <= 16 && S <= nk; ++S) {
+      const int64_t waves = (ntiles * S + sms - 1) / sms, w = bn / 128;
+      // products at 128 columns run at about 3/4 of the rate
+      const int64_t blocks = int64_t((nk + S - 1) / S) * (bn == 256 ? 6 : 4);
+      const int64_t c = waves * (blocks + 8) + (S > 1 ? (waves + S) * 2 * w : 0);
+      if (cost < 0 || c < cost) {
+        cost = c;
+        best = Shape32{bn, S};
+      }
     }
   }
   return best;
