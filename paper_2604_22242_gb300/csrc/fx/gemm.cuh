@@ -299,10 +299,30 @@ template <class T, int NIN, class Root> struct umma_ok {
   }();
 };
 
-// Evaluates the whole tree with umma::k_gemm_umma when the operands allow
-// TMA (16-byte aligned bases and leading dimensions) and the shapes agree;
-// *used is false otherwise (the caller takes the library-GEMM path, which
-// also reports shape errors).
+// Do two bound matrices of `es`-byte elements share memory (as whole spans)?
+inline bool overlap(const Binding& x, const Binding& y, size_t es) {
+  auto span = [es](const Binding& b) { return (size_t(b.ld) * size_t(b.cols - 1) + size_t(b.rows)) * es; };
+  const uintptr_t p = reinterpret_cast<uintptr_t>(x.p), q = reinterpret_cast<uintptr_t>(y.p);
+  return p < q + span(y) && q < p + span(x);
+}
+
+// Products from which copying unaligned 16-bit operands, and splitting FP32
+// ones, pays (M N K; any size with blocks_per_sm given). With the library's
+// GEMM and the pass after it on the other side: BF16 1001 x 301 x 1501 26.8
+// against 24.9 us, 513 x 7001 x 513 28.7 against 43.5, 1501^3 28.9 against
+// 61.7, 4001^3 190 against 850; FP32 257 x 3000 x 257 28.8 against 22.9,
+// 1000 x 300 x 1500 33 against 39, 1500^3 61 against 119, 3000^3 245 against
+// 858.
+constexpr double kRelayoutMin = double(1 << 30), kSplitMin = double(1 << 28);
+
+// Evaluates the whole tree with umma::k_gemm_umma. TMA wants 16-byte aligned
+// bases and leading dimensions; an operand without them is first copied to a
+// workspace that has (k_relayout16: 4 bytes moved per operand element, small
+// beside a large product, where the library's kernels for such operands run at
+// a fraction of the tensor cores' rate). *used is false when the shapes disagree (the caller's library
+// path reports it), for a bare or scaled product of unaligned operands
+// (nothing to fuse), when Z is written over an operand read in place beside
+// a copied one, or without workspace.
 template <class T, int NIN, class Root>
 fx_status run_umma(fx_expr* x, const Root& root, cudaStream_t st, bool* used) {
   *used = false;
@@ -332,10 +352,16 @@ fx_status run_umma(fx_expr* x, const Root& root, cudaStream_t st, bool* used) {
     return FX_OK;  // the library-GEMM path reports the shape error
   }
   CUtensorMap ma, mb;
-  const bool oka = AMN ? encode_map<T>(&ma, a.p, M, Ka, a.ld, 64, 64)
-                       : encode_map<T>(&ma, a.p, Ka, M, a.ld, 64, umma::BM);
-  const bool okb = BMN ? encode_map<T>(&mb, b.p, N, Ka, b.ld, 64, 64)
-                       : encode_map<T>(&mb, b.p, Ka, N, b.ld, 64, umma::BN);
+  const int sms = device_sms() > 0 ? device_sms() : 1;
+  // Pairs of CTAs where their 256 x 256 tiles fill the chip in no more waves
+  // than single CTAs' 128 x 256 ones do (8192^3 BF16: 683 us against 722)
+  const int64_t ntiles = ((M + umma::BM - 1) / umma::BM) * ((N + umma::BN - 1) / umma::BN);
+  const int64_t ptiles = ((M + umma::PBM - 1) / umma::PBM) * ((N + umma::BN - 1) / umma::BN);
+  const bool pair = (ptiles * 2 + sms - 1) / sms <= (ntiles + sms - 1) / sms && ptiles * 2 >= sms;
+  auto encode = [](CUtensorMap* m, const Binding& o, bool mn, int box) {
+    return encode_map<T>(m, o.p, o.rows, o.cols, o.ld, 64, mn ? 64 : box);
+  };
+  const bool oka = encode(&ma, a, AMN, umma::BM), okb = encode(&mb, b, BMN, pair ? umma::BN / 2 : umma::BN);
   if (!oka || !okb) return FX_OK;
   auto kern = umma::k_gemm_umma<T, AMN, BMN, Lifted, PS>;
   const int smem = umma::NS * umma::STAGE + 1024 + int(sizeof(umma::Bars));
@@ -343,24 +369,45 @@ fx_status run_umma(fx_expr* x, const Root& root, cudaStream_t st, bool* used) {
   FX_TRY(x->ws_err.ensure(256, st));
   unsigned int* err = static_cast<unsigned int*>(x->ws_err.p);
   const Slots sl = make_slots(x->b, NIN);
-  const int64_t ntiles = ((M + umma::BM - 1) / umma::BM) * ((N + umma::BN - 1) / umma::BN);
-  const int sms = device_sms() > 0 ? device_sms() : 1;
   const unsigned grid = unsigned(ntiles < sms ? ntiles : sms);   // persistent: one CTA per SM
   *used = true;
   x->last_launches = 0;
-  kern<<<grid, 192, smem, st>>>(ma, mb, LR::make(root), sl, static_cast<T*>(zb.p), zb.ld, int(M),
+  if (pair) {
+    auto pk = umma::k_gemm_umma_pair<T, AMN, BMN, Lifted, PS>;
+    const int psmem = umma::PNS * umma::PSTAGE + 1024 + int(sizeof(umma::PairBars));
+    FX_TRY(allow_smem(pk, psmem));
+    // as many pairs as can be resident: a tile processor may have an SM without a partner
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(unsigned(sms / 2 * 2));
+    cfg.blockDim = dim3(umma::THREADS);
+    cfg.dynamicSmemBytes = size_t(psmem);
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int pairs = 0;
+    if (cudaOccupancyMaxActiveClusters(&pairs, pk, &cfg) != cudaSuccess || pairs < 1) {
+      cudaGetLastError();
+      pairs = 1;
+    }
+    if (pairs > sms / 2) pairs = sms / 2;
+    if (pairs > ptiles) pairs = int(ptiles);
+    pk<<<unsigned(2 * pairs), umma::THREADS, psmem, st>>>(ma, mb, LR::make(root), sl, static_cast<T*>(zb.p), zb.ld,
+                                                int(M), int(N), int(Ka), err);
+    const cudaError_t pe = cudaGetLastError();
+    if (pe != cudaSuccess) return cuda_fail(pe, "k_gemm_umma_pair");
+    x->last_launches = 1;
+    return FX_OK;
+  }
+  kern<<<grid, umma::THREADS, smem, st>>>(ma, mb, LR::make(root), sl, static_cast<T*>(zb.p), zb.ld, int(M),
                                 int(N), int(Ka), err);
   const cudaError_t le = cudaGetLastError();
   if (le != cudaSuccess) return cuda_fail(le, "k_gemm_umma");
   x->last_launches = 1;
   return FX_OK;
-}
-
-// Do two bound matrices of `es`-byte elements share memory (as whole spans)?
-inline bool overlap(const Binding& x, const Binding& y, size_t es) {
-  auto span = [es](const Binding& b) { return (size_t(b.ld) * size_t(b.cols - 1) + size_t(b.rows)) * es; };
-  const uintptr_t p = reinterpret_cast<uintptr_t>(x.p), q = reinterpret_cast<uintptr_t>(y.p);
-  return p < q + span(y) && q < p + span(x);
 }
 
 // FP32: the operands split into BF16 planes, then umma32::k_gemm_umma32 (two
@@ -388,6 +435,7 @@ fx_status run_umma32(fx_expr* x, const Root& root, cudaStream_t st, bool* used) 
   if (K != Kb || zb.rows != M || zb.cols != N || M == 0 || N == 0 || K == 0) return FX_OK;
   const int64_t lim = int64_t(1) << 30;
   if (M >= lim || N >= lim || K >= lim) return FX_OK;
+  if (double(M) * double(N) * double(K) < kSplitMin && x->tune.bps == 0) return FX_OK;
   // Z written over an operand: the fallback for unsplittable values reads the
   // operands while other blocks store
   if (overlap(zb, a, sizeof(float)) || overlap(zb, b, sizeof(float))) return FX_OK;

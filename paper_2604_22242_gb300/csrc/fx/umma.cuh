@@ -11,7 +11,7 @@
 // lifted tree, in which P is a leaf - element by element, reading the other
 // leaves (W) from global memory and writing Z once.
 //
-// Persistent: one CTA of 192 threads per SM walks the output tiles (in
+// Persistent: one CTA of 320 threads per SM walks the output tiles (in
 // groups of 16 tile rows, for L2 reuse of the operands):
 //   warp 0      lane 0 loads the operand tiles with TMA (cp.async.bulk.tensor,
 //               128-byte swizzle) into a ring of NS shared-memory stages,
@@ -23,12 +23,16 @@
 //               have read it); after the tile's last step it commits to the
 //               accumulator's "full" barrier, and before reusing an
 //               accumulator it waits until the epilogue has read it out;
-//   warps 2..5  wait for a tile's accumulator, load their 32 TMEM lanes
-//               (rows) 16 columns at a time (tcgen05.ld 32x32b), release the
+//   warps 2..9  load the other leaves' values of their first columns, wait
+//               for a tile's accumulator, load 32 TMEM lanes (rows) of half
+//               its columns 32 at a time (tcgen05.ld 32x32b), release the
 //               accumulator after the last load, evaluate the remainder and
 //               store - while the next tile is multiplied into the other
-//               accumulator. The other leaves' values for the next 16
-//               columns are loaded before the current ones are computed.
+//               accumulator.
+// Products with many tiles run on pairs of CTAs (k_gemm_umma_pair below).
+// sigmoid(s X Y + W): BF16 8192^3 728 us with four epilogue warps that loaded
+// one piece of 16 columns ahead, 722 with these, 683 in pairs; 2000 x 1000 x
+// 1000 30.9 and 22.7 us.
 //
 // Operand layouts: column-major storage makes an operand K-major (K
 // contiguous) when it is read transposed or is the right factor, and
@@ -106,7 +110,7 @@ FX_D void commit(uint64_t* bar) {
 }
 FX_D void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 FX_D void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// 16 consecutive FP32 columns of this thread's TMEM lane (warp-wide).
+// 16 or 32 consecutive FP32 columns of this thread's TMEM lane (warp-wide).
 FX_D void ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
@@ -114,6 +118,18 @@ FX_D void ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
         "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
         "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+FX_D void ld32(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
+      "%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]),
+        "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
+        "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr)
       : "memory");
 }
@@ -193,7 +209,56 @@ FX_D void tile_of(int t, int tiles_m, int tiles_n, int& tm, int& tn) {
   tn = within / gsize;
 }
 
-constexpr int CW = 16;   // epilogue columns per TMEM load
+constexpr int CW = 32;         // epilogue columns per TMEM load
+constexpr int EPI_WARPS = 8;   // two per TMEM lane quarter
+constexpr int EC = BN / 2;     // columns each reads
+constexpr int THREADS = 64 + 32 * EPI_WARPS;
+
+// A thread's row m of Z, columns n0 .. n0 + EC - 1, from its TMEM lane at
+// taddr. The other leaves' values of the first two pieces of 32 columns are
+// loaded before wait() (the tile's products are still running) and each later
+// one two pieces ahead: at 16 columns one ahead, in four warps, a tile's
+// epilogue was a chain of 16 loads from memory, about 16 us that only a long
+// product hid. read_out() runs once the accumulator has been read
+// (warp-uniform); false when wait() gives up.
+template <class T, class E, int PS, class W, class F>
+FX_D bool epilogue_rows(const E& e, const Slots& sl, T* z, int64_t ldz, int64_t m, int M, int n0, int N,
+                        uint32_t taddr, const W& wait, const F& read_out) {
+  using LL = leaves_t<E>;
+  constexpr int NL = tl_size<LL>::value;
+  const bool row = m < M;
+  T w[2][NL][CW];
+  auto load = [&](int b, int n) {
+    if (row && n < N) load_others<LL, PS, T, CW>(w[b], sl, m, n, N - n < CW ? N - n : CW);
+  };
+  load(0, n0);
+  load(1, n0 + CW);
+  if (!wait()) return false;
+#pragma unroll
+  for (int c = 0; c < EC / CW; ++c) {
+    const int nc = n0 + c * CW;
+    uint32_t r[CW];
+    ld32(taddr + uint32_t(c * CW), r);
+    wait_ld();
+    if (c == EC / CW - 1) {  // the accumulator buffer is free for the MMA warp
+      fence_before();
+      __syncwarp();
+      read_out();
+    }
+    if (nc >= N) continue;  // warp-uniform
+    if (row) {
+#pragma unroll
+      for (int j = 0; j < CW; ++j) {
+        if (j < N - nc) {
+          ECtx<LL, PS, T, CW> cx{w[c & 1], __uint_as_float(r[j]), j};
+          sstore(z + m + int64_t(nc + j) * ldz, narrow_to<T>::from(e.ev(cx)));
+        }
+      }
+    }
+    if (c + 2 < EC / CW) load(c & 1, nc + 2 * CW);
+  }
+  return true;
+}
 
 // Z (M x N, column-major, ldz) = E(P) with P = op(A) op(B) of K terms, on a
 // persistent grid: CTA b takes tiles b, b + gridDim.x, ... The MMA warp
@@ -202,12 +267,10 @@ constexpr int CW = 16;   // epilogue columns per TMEM load
 // AMN / BMN: the A / B tiles are MN-major (else K-major). PS: the slot of
 // the product leaf in E.
 template <class T, bool AMN, bool BMN, class E, int PS>
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(THREADS, 1)
     k_gemm_umma(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                 const E e, const Slots sl, T* z, const int64_t ldz, const int M, const int N,
                 const int K, unsigned int* err) {
-  using LL = leaves_t<E>;
-  constexpr int NL = tl_size<LL>::value;
   extern __shared__ char smem_raw[];
   char* smem = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                        ~uintptr_t(1023));
@@ -223,7 +286,7 @@ __global__ void __launch_bounds__(192, 1)
     }
     for (int b = 0; b < 2; ++b) {
       tma::mbar_init(&bars.accf[b], 1);
-      tma::mbar_init(&bars.acce[b], 4);
+      tma::mbar_init(&bars.acce[b], EPI_WARPS);
     }
     tma::mbar_init(&bars.drain, 1);
     bars.abort = 0;
@@ -338,52 +401,25 @@ __global__ void __launch_bounds__(192, 1)
       tma::wait(&bars.drain, 0u, err);
     }
     __syncwarp();
-  } else {  // epilogue: warps 2..5 take TMEM lane quarters 2, 3, 0, 1
-    const int q = warp & 3;
+  } else {  // epilogue: warp w takes TMEM lane quarter w % 4 and half of the columns
+    const int q = warp & 3, col = (warp - 2) / 4 * EC;
     int i = 0;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
       const int b = i & 1;
-      const bool ready = tma::wait(&bars.accf[b], uint32_t(i / 2) & 1u, err);
-      fence_after();
-      // the TMEM loads below are warp-wide: the warp decides together
-      if (!__all_sync(0xffffffffu, ready && !bars.abort)) break;
       int tm, tn;
       tile_of(t, tiles_m, tiles_n, tm, tn);
-      const int64_t m = int64_t(tm) * BM + q * 32 + lane;
-      const int n0 = tn * BN;
-      const bool row = m < M;
-      T wn[NL][CW], wc[NL][CW];
-      if (row) load_others<LL, PS, T, CW>(wn, sl, m, n0, N - n0 < CW ? N - n0 : CW);
-#pragma unroll 1
-      for (int c = 0; c < BN / CW; ++c) {
-        const int nc = n0 + c * CW;
-        uint32_t r[CW];
-        ld16(tbase + uint32_t(b * BN) + (uint32_t(q * 32) << 16) + uint32_t(c * CW), r);
-        wait_ld();
-        if (c == BN / CW - 1) {  // the accumulator buffer is free for the MMA warp
-          fence_before();
-          __syncwarp();
-          if (lane == 0) tma::arrive(&bars.acce[b]);
-        }
-        if (nc >= N) continue;  // warp-uniform
-        const int nn = N - nc < CW ? N - nc : CW;
-#pragma unroll
-        for (int l = 0; l < NL; ++l)
-#pragma unroll
-          for (int j = 0; j < CW; ++j) wc[l][j] = wn[l][j];
-        const int nx = nc + CW;
-        if (row && c + 1 < BN / CW && nx < N)
-          load_others<LL, PS, T, CW>(wn, sl, m, nx, N - nx < CW ? N - nx : CW);
-        if (row) {
-#pragma unroll
-          for (int j = 0; j < CW; ++j) {
-            if (j < nn) {
-              ECtx<LL, PS, T, CW> cx{wc, __uint_as_float(r[j]), j};
-              sstore(z + m + int64_t(nc + j) * ldz, narrow_to<T>::from(e.ev(cx)));
-            }
-          }
-        }
-      }
+      auto wait = [&]() {
+        const bool ready = tma::wait(&bars.accf[b], uint32_t(i / 2) & 1u, err);
+        fence_after();
+        // the TMEM loads are warp-wide: the warp decides together
+        return bool(__all_sync(0xffffffffu, ready && !bars.abort));
+      };
+      auto read_out = [&]() {
+        if (lane == 0) tma::arrive(&bars.acce[b]);
+      };
+      if (!epilogue_rows<T, E, PS>(e, sl, z, ldz, int64_t(tm) * BM + q * 32 + lane, M, tn * BN + col, N,
+                                   tbase + uint32_t(b * BN + col) + (uint32_t(q * 32) << 16), wait, read_out))
+        break;
     }
   }
   fence_before();
@@ -391,6 +427,244 @@ __global__ void __launch_bounds__(192, 1)
   if (warp == 1) {
     fence_after();
     tmem_dealloc(tbase, TMEM_COLS);
+  }
+}
+
+// ---------------------------------------------------------------- CTA pairs
+//
+// k_gemm_umma_pair: the same product on clusters of two CTAs, whose SMs work
+// on one 256 x 256 tile (cta_group::2). Each CTA holds 128 rows of A and half
+// of B's 256 columns in shared memory, and 128 rows of the accumulator in its
+// TMEM; the leader's MMA thread issues for both, and each SM's tensor core
+// reads the other half of B from its peer. Per SM that is 16 + 16 KB a K
+// step instead of 16 + 32: a third less operand traffic from L2 and into
+// shared memory, and six stages instead of four in the same space.
+//
+//   full[s]   in the leader: the bytes of both CTAs' loads (a pair's loads may
+//             signal the peer's barrier) and the leader's own arrival
+//   empty[s]  in each CTA: the leader's commit, multicast to both
+//   accf[b]   in each CTA: likewise, once per tile
+//   acce[b]   in the leader: one arrival per epilogue warp of both CTAs
+//
+// A cluster barrier after the set-up (barriers exist before a peer signals
+// them) and one before the TMEM is freed and the CTAs leave; every thread
+// reaches both, since all other waits are bounded.
+constexpr int PBM = 256, PNS = 6, PSTAGE = 2 * SA;  // A and B halves: 128 x 64 each
+
+FX_D uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// Shared-memory address of `p` in the CTA of rank `rank` of this cluster.
+FX_D uint32_t peer_addr(const void* p, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(tma::saddr(p)), "r"(rank));
+  return r;
+}
+FX_D void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+FX_D void remote_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+FX_D void remote_store(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+FX_D void pair_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3}], [%4];" ::"r"(tma::saddr(dst)),
+      "l"(map), "r"(x), "r"(y), "r"(bar)
+      : "memory");
+}
+FX_D void pair_alloc(uint32_t* slot, uint32_t ncols) {
+  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tma::saddr(slot)),
+               "r"(ncols)
+               : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+FX_D void pair_dealloc(uint32_t taddr, uint32_t ncols) {
+  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+FX_D void pair_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
+  asm volatile(
+      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
+      "l"(a), "l"(b), "r"(id), "r"(acc)
+      : "memory");
+}
+// Arrive on `bar` (at its offset in both CTAs) once this thread's MMAs are done.
+FX_D void pair_commit(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+          tma::saddr(bar)),
+      "h"(uint16_t(3))
+      : "memory");
+}
+template <class T, bool AMN, bool BMN> FX_HD constexpr uint32_t pair_idesc() {
+  constexpr uint32_t fmt = std::is_same<T, bf16>::value ? 1u : 0u;
+  return (1u << 4) | (fmt << 7) | (fmt << 10) | (uint32_t(AMN) << 15) | (uint32_t(BMN) << 16) |
+         (uint32_t(BN >> 3) << 17) | (uint32_t(PBM >> 4) << 24);
+}
+
+struct PairBars {
+  uint64_t full[PNS], empty[PNS];
+  uint64_t accf[2], acce[2];
+  uint64_t drain;
+  uint32_t taddr;
+  volatile uint32_t abort;
+};
+
+// 128 rows of an operand's K block into 16 KB at dst.
+template <bool MNMAJOR> FX_D void pair_load_half(char* dst, const CUtensorMap* m, int mn0, int k0, uint32_t bar) {
+  if (MNMAJOR) {
+    pair_load_2d(dst, m, mn0, k0, bar);
+    pair_load_2d(dst + SA / 2, m, mn0 + 64, k0, bar);
+  } else {
+    pair_load_2d(dst, m, k0, mn0, bar);
+  }
+}
+
+template <class T, bool AMN, bool BMN, class E, int PS>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
+    k_gemm_umma_pair(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
+                     const E e, const Slots sl, T* z, const int64_t ldz, const int M, const int N,
+                     const int K, unsigned int* err) {
+  extern __shared__ char smem_raw[];
+  char* smem = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                       ~uintptr_t(1023));
+  PairBars& bars = *reinterpret_cast<PairBars*>(smem + PNS * PSTAGE);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const uint32_t rank = cluster_rank();
+  const int tiles_m = (M + PBM - 1) / PBM, tiles_n = (N + BN - 1) / BN;
+  const int ntiles = tiles_m * tiles_n;
+  const int first = int(blockIdx.x) / 2, step = int(gridDim.x) / 2;
+  const int nk = (K + BK - 1) / BK;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < PNS; ++s) {
+      tma::mbar_init(&bars.full[s], 1);
+      tma::mbar_init(&bars.empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      tma::mbar_init(&bars.accf[b], 1);
+      tma::mbar_init(&bars.acce[b], 2 * EPI_WARPS);
+    }
+    tma::mbar_init(&bars.drain, 1);
+    bars.abort = 0;
+    tma::fence_mbar_init();
+  }
+  __syncthreads();
+  cluster_sync();
+  if (warp == 1) pair_alloc(&bars.taddr, TMEM_COLS);
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tbase = bars.taddr;
+  auto give_up = [&]() {  // both CTAs' epilogues see it
+    remote_store(peer_addr(const_cast<uint32_t*>(&bars.abort), 0), 1u);
+    remote_store(peer_addr(const_cast<uint32_t*>(&bars.abort), 1), 1u);
+  };
+
+  if (warp == 0) {
+    if (lane == 0) {
+      uint32_t g = 0;
+      bool ok = true;
+      for (int t = first; t < ntiles && ok; t += step) {
+        int tm, tn;
+        tile_of(t, tiles_m, tiles_n, tm, tn);
+        const int m0 = tm * PBM + int(rank) * BM, n0 = tn * BN + int(rank) * (BN / 2);
+        for (int kt = 0; kt < nk; ++kt, ++g) {
+          const int s = int(g % PNS);
+          if (g >= uint32_t(PNS) && !tma::wait(&bars.empty[s], ((g - PNS) / PNS) & 1u, err)) {
+            ok = false;
+            break;
+          }
+          if (rank == 0) tma::arrive_expect_tx(&bars.full[s], 2 * PSTAGE);
+          const uint32_t bar = peer_addr(&bars.full[s], 0);
+          char* st = smem + s * PSTAGE;
+          pair_load_half<AMN>(st, &mapA, m0, kt * BK, bar);
+          pair_load_half<BMN>(st + SA, &mapB, n0, kt * BK, bar);
+        }
+      }
+      if (!ok) {  // the leader waits (bounded) for the copies still in flight
+        give_up();
+        if (rank == 0)
+          for (uint32_t j = (g > uint32_t(PNS) ? g - PNS : 0); j < g; ++j)
+            tma::wait(&bars.full[j % PNS], (j / PNS) & 1u, nullptr);
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    if (lane == 0 && rank == 0) {
+      constexpr uint32_t ID = pair_idesc<T, AMN, BMN>();
+      uint32_t g = 0;
+      int i = 0;
+      bool ok = true;
+      for (int t = first; t < ntiles && ok; t += step, ++i) {
+        const int b = i & 1;
+        if (i >= 2 && !tma::wait(&bars.acce[b], uint32_t((i - 2) / 2) & 1u, err)) {
+          ok = false;
+          break;
+        }
+        fence_after();
+        const uint32_t tacc = tbase + uint32_t(b * BN);
+        for (int kt = 0; kt < nk; ++kt, ++g) {
+          const int s = int(g % PNS);
+          if (!tma::wait(&bars.full[s], (g / PNS) & 1u, err)) {
+            ok = false;
+            break;
+          }
+          fence_after();
+          const uint32_t sa = tma::saddr(smem + s * PSTAGE), sb = sa + SA;
+#pragma unroll
+          for (int k = 0; k < BK / UK; ++k) {
+            const uint64_t ad = AMN ? desc(sa + k * UK * 128, SA / 2, 1024) : desc(sa + k * UK * 2, 16, 1024);
+            const uint64_t bd = BMN ? desc(sb + k * UK * 128, SA / 2, 1024) : desc(sb + k * UK * 2, 16, 1024);
+            pair_mma(tacc, ad, bd, ID, (kt > 0 || k > 0) ? 1u : 0u);
+          }
+          pair_commit(&bars.empty[s]);
+        }
+        if (ok) pair_commit(&bars.accf[b]);
+      }
+      if (!ok) {
+        give_up();
+        pair_commit(&bars.accf[0]);
+        pair_commit(&bars.accf[1]);
+      }
+      pair_commit(&bars.drain);
+    }
+    // both CTAs: no product, and no commit to this CTA's barriers, is in flight
+    if (lane == 0) tma::wait(&bars.drain, 0u, err);
+    __syncwarp();
+  } else {
+    const int q = warp & 3, col = (warp - 2) / 4 * EC;
+    int i = 0;
+    for (int t = first; t < ntiles; t += step, ++i) {
+      const int b = i & 1;
+      int tm, tn;
+      tile_of(t, tiles_m, tiles_n, tm, tn);
+      const uint32_t acce = peer_addr(&bars.acce[b], 0);
+      auto wait = [&]() {
+        const bool ready = tma::wait(&bars.accf[b], uint32_t(i / 2) & 1u, err);
+        fence_after();
+        return bool(__all_sync(0xffffffffu, ready && !bars.abort));
+      };
+      auto read_out = [&]() {
+        if (lane == 0) remote_arrive(acce);
+      };
+      if (!epilogue_rows<T, E, PS>(e, sl, z, ldz, int64_t(tm) * PBM + rank * BM + q * 32 + lane, M,
+                                   tn * BN + col, N,
+                                   tbase + uint32_t(b * BN + col) + (uint32_t(q * 32) << 16), wait, read_out))
+        break;
+    }
+  }
+  fence_before();
+  __syncthreads();
+  cluster_sync();
+  if (warp == 1) {
+    fence_after();
+    pair_dealloc(tbase, TMEM_COLS);
   }
 }
 
