@@ -362,7 +362,33 @@ fx_status run_umma(fx_expr* x, const Root& root, cudaStream_t st, bool* used) {
     return encode_map<T>(m, o.p, o.rows, o.cols, o.ld, 64, mn ? 64 : box);
   };
   const bool oka = encode(&ma, a, AMN, umma::BM), okb = encode(&mb, b, BMN, pair ? umma::BN / 2 : umma::BN);
-  if (!oka || !okb) return FX_OK;
+  umma::Relayout ca{}, cb{};
+  if (!oka || !okb) {
+    if (ScaledProd<Root>::value || (double(M) * double(N) * double(Ka) < kRelayoutMin && x->tune.bps == 0)) return FX_OK;
+    if ((oka && overlap(zb, a, sizeof(T))) || (okb && overlap(zb, b, sizeof(T)))) return FX_OK;
+    auto ldp = [](const Binding& o) { return (o.rows + 7) / 8 * 8; };
+    auto bytes = [&](const Binding& o) { return (size_t(ldp(o)) * size_t(o.cols) * sizeof(T) + 255) & ~size_t(255); };
+    auto copy = [&](const Binding& o, char* d) {
+      const int64_t pc = (o.rows + 255) / 256;
+      return umma::Relayout{o.p, d, o.rows, o.cols, o.ld, ldp(o), pc * o.cols, FastDiv::make(uint32_t(pc))};
+    };
+    const size_t na = oka ? 0 : bytes(a), nb = okb ? 0 : bytes(b);
+    if (x->ws_gemm.ensure(na + nb, st) != FX_OK) {
+      cudaGetLastError();
+      return FX_OK;
+    }
+    char* w = static_cast<char*>(x->ws_gemm.p);
+    auto moved = [&](const Binding& o, char* d) { return Binding{d, o.rows, o.cols, ldp(o), true}; };
+    if (!oka) {
+      ca = copy(a, w);
+      if (!encode(&ma, moved(a, w), AMN, umma::BM)) return FX_OK;
+    }
+    if (!okb) {
+      cb = copy(b, w + na);
+      if (!encode(&mb, moved(b, w + na), BMN, pair ? umma::BN / 2 : umma::BN)) return FX_OK;
+    }
+    if (ca.items >= (int64_t(1) << 32) || cb.items >= (int64_t(1) << 32)) return FX_OK;
+  }
   auto kern = umma::k_gemm_umma<T, AMN, BMN, Lifted, PS>;
   const int smem = umma::NS * umma::STAGE + 1024 + int(sizeof(umma::Bars));
   FX_TRY(allow_smem(kern, smem));
@@ -372,6 +398,12 @@ fx_status run_umma(fx_expr* x, const Root& root, cudaStream_t st, bool* used) {
   const unsigned grid = unsigned(ntiles < sms ? ntiles : sms);   // persistent: one CTA per SM
   *used = true;
   x->last_launches = 0;
+  if (ca.items + cb.items > 0) {
+    const int64_t blocks = (ca.items + cb.items + 7) / 8;
+    umma::k_relayout16<<<unsigned(blocks < sms * 8 ? blocks : sms * 8), 256, 0, st>>>(ca, cb);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(e, "k_relayout16");
+  }
   if (pair) {
     auto pk = umma::k_gemm_umma_pair<T, AMN, BMN, Lifted, PS>;
     const int psmem = umma::PNS * umma::PSTAGE + 1024 + int(sizeof(umma::PairBars));

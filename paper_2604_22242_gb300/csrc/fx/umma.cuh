@@ -668,6 +668,36 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   }
 }
 
+// A column-major 16-bit matrix of any base and leading dimension copied to
+// one that TMA can address (ldp a multiple of 8). A warp takes 256
+// consecutive elements of a column, 2 bytes per lane and access, so every
+// access of the warp is one 64-byte run whatever the alignment.
+struct Relayout {
+  const void* src;
+  void* dst;
+  int64_t d0, d1, ld, ldp;
+  int64_t items;     // 256-element pieces: ceil(d0 / 256) * d1 (0: nothing to copy)
+  FastDiv per_col;
+};
+static __global__ void __launch_bounds__(256) k_relayout16(const Relayout a, const Relayout b) {
+  const int lane = threadIdx.x % 32;
+  const int64_t n = a.items + b.items;
+  for (int64_t i = int64_t(blockIdx.x) * 8 + threadIdx.x / 32; i < n; i += int64_t(gridDim.x) * 8) {
+    const Relayout& o = i < a.items ? a : b;
+    const uint32_t q = uint32_t(i < a.items ? i : i - a.items);
+    const uint32_t c = o.per_col.div(q);
+    const int64_t r = int64_t(q - c * o.per_col.d) * 256 + lane;
+    const uint16_t* s = static_cast<const uint16_t*>(o.src) + r + int64_t(c) * o.ld;
+    uint16_t* d = static_cast<uint16_t*>(o.dst) + r + int64_t(c) * o.ldp;
+    uint16_t w[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) w[j] = r + 32 * j < o.d0 ? __ldg(s + 32 * j) : uint16_t(0);
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (r + 32 * j < o.d0) d[32 * j] = w[j];
+  }
+}
+
 }  // namespace umma
 
 // ---------------------------------------------------------------- host side
