@@ -368,16 +368,16 @@ __global__ void __launch_bounds__(NT) k_batch_async(const E e, const BatchMat* _
 //
 // k_batch_skew: the batch's tiles through skew_tile (skew.cuh): plain leaves
 // and Z as aligned 16-byte register vectors, transposed leaves as aligned
-// pieces staged in shared memory, two blocks of 512 threads per
-// SM (three of 256 for 2-byte types). The
+// pieces staged in shared memory, two blocks of 256 threads per
+// SM (three for 2-byte types). The
 // cp.async kernel above copies transposed leaves element by element and has
-// room for one block per SM (4096 matrices FP32: 3526 us, against 2618 with
+// room for one block per SM (4096 matrices FP32: 3517 us, against 2372 with
 // this one and the block-wide combine below); it stays for batches in which a matrix's plain
 // leaves and Z do not share their misalignment, and as launch-shape pipeline 1.
 //
-// Warp 0 reads the next item's descriptor, one 8-byte word per lane, while
-// the current tile loads, and the item after that, so that no tile waits for
-// a chain of dependent loads.
+// Warp 0 reads descriptors two items ahead, one 8-byte word per lane, while
+// the current tile loads, so that no tile waits for a chain of dependent
+// loads, and the next tile's lines can be prefetched.
 template <int NIN> struct SkewMat {  // the words of BatchMat that a tile needs
   const void* p[NIN + 1];
   int64_t ld[NIN + 1];
@@ -394,14 +394,19 @@ template <int NIN> FX_D int skew_word(int w) {
   constexpr int F = FX_MAX_SLOTS;
   return w <= NIN ? w : (w < 2 * NIN + 2 ? F + w - NIN - 1 : 2 * F + w - 2 * NIN - 2);
 }
-template <int NIN> struct SkewNext {
-  uint64_t* word;
+template <class SS, class T, int NIN> struct SkewNext {
+  uint64_t* word;                // the item after next: its descriptor arrives now
   BatchTile* tile;
   uint64_t w;
   BatchTile t;
+  const SkewMat<NIN>* m;         // the next item (null: none), whose lines are prefetched
+  const BatchTile* at;
   FX_D void operator()() const {
     if (threadIdx.x < sizeof(SkewMat<NIN>) / 8) word[threadIdx.x] = w;
     if (threadIdx.x == 0) *tile = t;
+    if (m)
+      skew_prefetch<SS, T>(MatSlots{m->p, m->ld}, SkewPlace{int(m->rows), int(m->cols), at->tr * SS::TR,
+                                                            at->tc * SS::TC, m->csbase, m->csld});
   }
 };
 // Stores a tile's values and adds them to the thread's sum.
@@ -433,7 +438,7 @@ template <class T, int KIND, class CT> struct SkewPut {
 };
 
 template <class E, class T, int V, int TR, int TC, int NT, int KIND, int NIN>
-__global__ void __launch_bounds__(NT, skew_blocks(NT))
+__global__ void __launch_bounds__(NT, skew_blocks<T>())
     k_batch_skew(const E e, const BatchMat* __restrict__ mats, const BatchTile* __restrict__ tiles,
                  const int64_t ntiles, double2* part) {
   using SS = SkewShape<E, T, V, TR, TC, NT>;
@@ -441,8 +446,8 @@ __global__ void __launch_bounds__(NT, skew_blocks(NT))
   constexpr int NWORD = int(sizeof(SkewMat<NIN>) / 8);
   static_assert(NWORD <= 32 && sizeof(SkewMat<NIN>) % 8 == 0, "one word per lane of warp 0");
   __shared__ CT sm[SS::SMEM];
-  __shared__ uint64_t words[2][NWORD];
-  __shared__ BatchTile at[2];
+  __shared__ uint64_t words[3][NWORD];
+  __shared__ BatchTile at[3];
   const int64_t G = gridDim.x;
   const int64_t last = ntiles - 1;
   auto item = [&](int64_t i) { return tiles[i < ntiles ? i : last]; };
@@ -450,22 +455,30 @@ __global__ void __launch_bounds__(NT, skew_blocks(NT))
     const int w = int(threadIdx.x) < NWORD ? int(threadIdx.x) : 0;
     return __ldg(reinterpret_cast<const unsigned long long*>(mats + t.mat) + skew_word<NIN>(w));
   };
+  auto put = [&](int b, const BatchTile& t) {
+    const uint64_t w = word(t);
+    if (threadIdx.x < NWORD) words[b][threadIdx.x] = w;
+    if (threadIdx.x == 0) at[b] = t;
+  };
   BatchTile next = {};
   if (threadIdx.x < 32) {
-    const BatchTile t0 = item(blockIdx.x);
-    SkewNext<NIN>{words[0], &at[0], word(t0), t0}();
-    next = item(blockIdx.x + G);
+    put(0, item(blockIdx.x));
+    put(1, item(blockIdx.x + G));
+    next = item(blockIdx.x + 2 * G);
   }
   __syncthreads();
   int b = 0;
-  for (int64_t i = blockIdx.x; i < ntiles; i += G, b ^= 1) {
+  for (int64_t i = blockIdx.x; i < ntiles; i += G) {
+    const int b1 = b == 2 ? 0 : b + 1, b2 = b1 == 2 ? 0 : b1 + 1;
     const SkewMat<NIN>& m = *reinterpret_cast<const SkewMat<NIN>*>(words[b]);
     const BatchTile t = at[b];
-    SkewNext<NIN> fetched{words[b ^ 1], &at[b ^ 1], 0, next};
+    SkewNext<SS, T, NIN> fetched{words[b2], &at[b2], 0, next, i + G < ntiles
+                                     ? reinterpret_cast<const SkewMat<NIN>*>(words[b1]) : nullptr, &at[b1]};
     if (threadIdx.x < 32) {
       fetched.w = word(next);
-      next = item(i + 2 * G);
+      next = item(i + 3 * G);
     }
+    b = b1;
     CT tsum = CT(0);  // a thread adds at most TR * TC / NT values of a tile
     const SkewPlace place{int(m.rows), int(m.cols), t.tr * TR, t.tc * TC, m.csbase, m.csld};
     T* z = static_cast<T*>(const_cast<void*>(m.p[NIN])) + (place.r0 + place.c0 * m.ld[NIN]);
@@ -791,7 +804,7 @@ fx_status run_batch(fx_expr* x, const Root& root, int64_t n, const fx_batch_item
     using B2 = std::integral_constant<int, 2>;
     using B3 = std::integral_constant<int, 3>;
     using B4 = std::integral_constant<int, 4>;
-    constexpr int SNT = skew_threads<T>();
+    constexpr int SNT = skew_threads();
     auto launch_skew = [&]() -> fx_status {
       if constexpr (V > 1 && V * sizeof(T) == 16 && tma_uniform<LL, T>()) {
         constexpr int KE = kind == FX_KIND_MULTI ? FX_KIND_MULTI : KIND0;

@@ -490,7 +490,7 @@ fx_status launch_tile_skew(const Run& r, const E& e, const Slots& sl, int64_t R,
     const int64_t lim = (int64_t(1) << 31) - 128;
     if (R >= lim || C >= lim || !skew_ok<LL, T, V>(r.b, z, epi.ldz, sbase, sld)) return FX_OK;
     using TC_ = TileCfg<E, V>;
-    constexpr int NT = skew_threads<T>();
+    constexpr int NT = skew_threads();
     auto kern = k_tile_skew<E, Epi, T, V, TC_::TR, TC_::TC, NT>;
     const int64_t tiles_r = (R + max_shift<V>(sbase, sld, C) + TC_::TR - 1) / TC_::TR;
     const int64_t ntiles = tiles_r * ((C + TC_::TC - 1) / TC_::TC);
