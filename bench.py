@@ -87,11 +87,10 @@ TRAFFIC = {
 }
 
 # FP64-pipe instructions per output element of FP64 trees (per lane: DFMA,
-# DADD and DMUL each take one slot), counted with ncu
-# (smsp__sass_thread_inst_executed_op_{dfma,dadd,dmul}_pred_on.sum over
-# 4096^2 elements): exp, sqrt and division of the Z tree run as FMA
-# sequences on the FP64 pipe, which on GB300 is slower than HBM.
-FP64_PIPE_OPS = {("expr8192_f64", "Z"): 35}
+# DADD and DMUL each take one slot): in the Z tree exp 4, sqrt 3, division 3
+# (fx/dmath.cuh), 1 + exp and the product's fma. The FP64 pipe is slower than
+# HBM on GB300.
+FP64_PIPE_OPS = {("expr8192_f64", "Z"): 12}
 
 
 def recorded_traffic(workload, dom, shape, source_hash):

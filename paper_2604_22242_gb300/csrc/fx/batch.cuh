@@ -4,10 +4,10 @@
 // (matrices in decreasing size order, so the smallest tiles come last and
 // fill the tail); one persistent launch (grid = SMs x resident blocks)
 // walks the list with a static stride and runs the same tile body as the
-// single-matrix tiled kernel (transposed leaves staged through shared
+// single-matrix skewed kernel (transposed leaves staged through shared
 // memory). A tree with an accu output writes one compensated partial per
-// warp of each tile; a second launch sums each matrix's partials in order
-// in FP64 (one warp per matrix). The list, the descriptors and both launches are
+// warp of each tile; a second launch sums each matrix's partials as pairs in
+// a fixed order (one block per matrix). The list, the descriptors and both launches are
 // cached per item array (kept as a copy and compared whole on the next call);
 // with use_graph the launches are captured once in a CUDA graph and replayed.
 #pragma once

@@ -9,7 +9,10 @@
 // plain leaf bound to that temporary, and the rest of the tree runs on the
 // fused path as usual. Two roots need no second pass: a bare product and a
 // scalar times a product (Fig. 1's Z = 2 X Y^T), whose scalar becomes the
-// GEMM's alpha and whose output is written straight into Z.
+// GEMM's alpha and whose output is written straight into Z. Trees with one
+// product of matrix leaves and an element-wise remainder run on the tensor
+// cores in one kernel instead (umma.cuh for BF16 and FP16, umma32.cuh for
+// FP32), where their sizes and operands allow it.
 //
 // Product operands must be matrix leaves, plain or transposed (a transpose
 // becomes the GEMM's operand op), or products themselves (the paper's
