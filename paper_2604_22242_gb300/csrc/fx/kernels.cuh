@@ -409,9 +409,11 @@ template <> struct MaxAcc<double, true> {
   long long m;
   FX_D void init() { m = -1; }
   // v is the abs node's operand: its magnitude is the pattern with the sign
-  // bit cleared (an integer and, not an FP64 instruction)
+  // bit cleared, word by word (an and of the whole 64-bit pattern is taken
+  // for fabs by the compiler, which makes it an FP64 instruction)
   FX_D void add(double v) {
-    const long long b = __double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFll;
+    const long long b = (static_cast<long long>(dm::hi_word(v) & 0x7FFFFFFFu) << 32) |
+                        static_cast<long long>(dm::lo_word(v));
     m = b > m ? b : m;
   }
   FX_D double get() const { return m < 0 ? neg_inf<double>() : __longlong_as_double(m); }
