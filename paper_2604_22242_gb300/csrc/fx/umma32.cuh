@@ -43,11 +43,15 @@
 // product's error against 64 bits is smaller (maximum of the result 8.7e-8
 // against 1.0e-7 at K = 2048, 9.0e-8 against 1.6e-7 at K = 700).
 //
-// Operands with an infinity, a NaN, a magnitude of 2^127 or more (it could
-// round up to a BF16 infinity) or a nonzero one below 2^-100 (its parts would
-// be subnormal) cannot be split this way: k_split3 records one in a flag and
-// every block then computes its tiles with FP32 fma from the operands
-// themselves. Every wait is bounded as in umma.cuh.
+// Operands with an infinity, a NaN, a magnitude of 2^60 or more or a nonzero
+// one below 2^-100 (its parts would be subnormal) are not computed this way:
+// k_split3 records one in a flag and every block then computes its tiles with
+// FP32 fma from the operands themselves. Below 2^60 a product is below 2^120
+// and a K block's 64 of them, with the small products, below 2^127, so the
+// accumulator stays finite: a1 b2 and a2 b1 have either sign, and one of them
+// at -Inf beside a1 b1 at +Inf would give NaN where FP32 gives an infinity.
+// What overflows later does so in the rounded FP32 adds, as in FP32. Every
+// wait is bounded as in umma.cuh.
 #pragma once
 
 #include "umma.cuh"
@@ -113,7 +117,7 @@ struct Bars {
 
 FX_D bool unsplittable(float a) {
   const uint32_t b = __float_as_uint(a) & 0x7FFFFFFFu;
-  return b - 0x0D800000u >= 0x7F000000u - 0x0D800000u && b != 0u;  // not in [2^-100, 2^127), not 0
+  return b - 0x0D800000u >= 0x5D800000u - 0x0D800000u && b != 0u;  // not in [2^-100, 2^60), not 0
 }
 
 struct SplitArgs {
