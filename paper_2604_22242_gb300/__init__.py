@@ -285,22 +285,32 @@ def bind_tensor(h, slot: int, t):
 # of them: (event recorded after those launches, handle). fx_expr_destroy
 # frees workspace without waiting for the kernels that use it, so a handle is
 # destroyed only once its event has completed; at most _RETIRED_MAX are held.
+# Finalizers end up here at any point, inside _retire itself included: they
+# add their handle (one atomic append) and leave the rest to whoever is at it,
+# so nobody waits for the lock. An entry is out of the list while its event is
+# asked or waited for and its handle destroyed.
 _retired = []
 _retired_lock = threading.Lock()
 _RETIRED_MAX = 32
 
 
 def _retire(event, h):
-    with _retired_lock:
-        _retired.append((event, h))
-        done = [e for e in _retired if e[0].query()]
-        _retired[:] = [e for e in _retired if e not in done]
+    _retired.append((event, h))
+    if not _retired_lock.acquire(blocking=False):
+        return
+    try:
+        for _ in range(len(_retired)):
+            e, x = _retired.pop(0)
+            if e.query():
+                fx_expr_destroy(x)
+            else:
+                _retired.append((e, x))
         while len(_retired) > _RETIRED_MAX:
-            e = _retired.pop(0)
-            e[0].synchronize()
-            done.append(e)
-    for _, x in done:
-        fx_expr_destroy(x)
+            e, x = _retired.pop(0)
+            e.synchronize()
+            fx_expr_destroy(x)
+    finally:
+        _retired_lock.release()
 
 
 class Expr:
