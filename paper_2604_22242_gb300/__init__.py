@@ -285,6 +285,9 @@ def bind_tensor(h, slot: int, t):
 # of them: (event recorded after those launches, handle). fx_expr_destroy
 # frees workspace without waiting for the kernels that use it, so a handle is
 # destroyed only once its event has completed; at most _RETIRED_MAX are held.
+# Without an event (launches recorded into a graph: there is nothing to ask) it
+# is destroyed as soon as its stream is not capturing: neither a query nor a
+# free may run during a capture, and neither is tried then.
 # Finalizers end up here at any point, inside _retire itself included: they
 # add their handle (one atomic append) and leave the rest to whoever is at it,
 # so nobody waits for the lock. An entry is out of the list while its event is
@@ -294,20 +297,26 @@ _retired_lock = threading.Lock()
 _RETIRED_MAX = 32
 
 
+def _capturing():
+    cuda = _torch().cuda
+    return cuda.is_initialized() and cuda.is_current_stream_capturing()
+
+
 def _retire(event, h):
     _retired.append((event, h))
-    if not _retired_lock.acquire(blocking=False):
+    if _capturing() or not _retired_lock.acquire(blocking=False):
         return
     try:
         for _ in range(len(_retired)):
             e, x = _retired.pop(0)
-            if e.query():
+            if e is None or e.query():
                 fx_expr_destroy(x)
             else:
                 _retired.append((e, x))
         while len(_retired) > _RETIRED_MAX:
             e, x = _retired.pop(0)
-            e.synchronize()
+            if e is not None:
+                e.synchronize()
             fx_expr_destroy(x)
     finally:
         _retired_lock.release()
@@ -316,7 +325,10 @@ def _retire(event, h):
 class Expr:
     """An expression object with its slots bound to torch tensors."""
 
-    _last = None  # event after the last launches; set where nobody else waits for them
+    # event after the last launches, where nobody else waits for them; None once
+    # marked: they were recorded into a graph
+    _last = None
+    _marked = False
 
     def __init__(self, name: str, storage: int):
         self.h = fx_expr_create(name, storage)
@@ -344,13 +356,15 @@ class Expr:
     def mark(self):
         """Notes that launches of this handle are in flight on the current
         stream: close() then destroys it only after they have finished."""
-        self._last = _torch().cuda.Event()
-        self._last.record()
+        self._marked, self._last = True, None
+        if not _capturing():
+            self._last = _torch().cuda.Event()
+            self._last.record()
 
     def close(self):
         if self.h:
             h, self.h = self.h, None
-            if self._last is None:
+            if self._last is None and not self._marked:
                 fx_expr_destroy(h)
             else:
                 _retire(self._last, h)

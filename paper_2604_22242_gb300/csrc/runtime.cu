@@ -100,8 +100,10 @@ fx_status Workspace::ensure(size_t need, cudaStream_t st) {
 
 void Workspace::release() {
   if (p) {
-    // The caller guarantees no launch of this object is in flight.
-    cudaFree(p);
+    // The caller guarantees no launch of this object is in flight. Memory
+    // allocated in a capture belongs to its graph and cannot be freed here:
+    // the refusal must not be left for the next launch's error check.
+    if (cudaFree(p) != cudaSuccess) cudaGetLastError();
   }
   p = nullptr;
   bytes = 0;
