@@ -634,8 +634,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       }
       pair_commit(&bars.drain);
     }
-    // both CTAs: no product, and no commit to this CTA's barriers, is in flight
-    if (lane == 0) tma::wait(&bars.drain, 0u, err);
+    // Both CTAs: no product, and no commit to this CTA's barriers, is in flight.
+    // The second CTA's wait lasts for the whole launch: the limit on polls
+    // counts per tile, as in every other wait.
+    if (lane == 0) {
+      bool done = false;
+      for (int t = first; t < ntiles && !done && !bars.abort; t += step)
+        done = tma::wait(&bars.drain, 0u, nullptr);
+      if (!done) tma::wait(&bars.drain, 0u, err);
+    }
     __syncwarp();
   } else {
     const int q = warp & 3, col = (warp - 2) / 4 * EC;
