@@ -251,6 +251,18 @@ FX_D void prefetch_others(const Slots& sl, int64_t m, int64_t n, int M) {
   }
 }
 
+// Barrier 1 over the block's NT epilogue threads; true if v is for all of them.
+template <int NT> FX_D bool all_of(bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbar.red.and.pred q, 1, %2, p;\n"
+      "selp.u32 %0, 1, 0, q;\n}"
+      : "=r"(r)
+      : "r"(uint32_t(v)), "n"(NT)
+      : "memory");
+  return r != 0;
+}
+
 // The product by FP32 fma from the operands themselves (unsplittable values):
 // 256 threads, 8 x 8 results each, K steps of 16 through shared memory.
 template <int BN, class E, int PS>
@@ -509,13 +521,17 @@ __global__ void __launch_bounds__(Slots32<BN>::THREADS, 1)
         __syncwarp();
         if (lane == 0) tma::arrive(&bars.acce[b]);
       }
-      if (!ready) break;
+      if (S == 1 && !ready) break;
       if (S > 1) {
         float* mine = part + int64_t(it) * (BM * BN) + col * BM + row;
+        if (ready) {
 #pragma unroll
-        for (int j = 0; j < NC; ++j) __stcg(mine + j * BM, acc[j]);
+          for (int j = 0; j < NC; ++j) __stcg(mine + j * BM, acc[j]);
+        }
         __threadfence();
-        asm volatile("bar.sync 1, %0;" ::"n"(32 * SL::EPI_WARPS) : "memory");
+        // a warp that gave up its wait still comes here: the warps leave
+        // together, and none is left at a barrier that another never reaches
+        if (!all_of<32 * SL::EPI_WARPS>(ready)) break;
         if (warp == 2 && lane == 0) bars.last = atomicAdd(tickets + t, 1u) == unsigned(S - 1);
         asm volatile("bar.sync 1, %0;" ::"n"(32 * SL::EPI_WARPS) : "memory");
         if (!bars.last) continue;
