@@ -151,7 +151,7 @@ FX_D void issue_tile(char* buf, const IssueDesc<NIN>& d) {
     using T = typename L::elem;
     T* dst = reinterpret_cast<T*>(buf + abuf_offset<LL, TR, TC, I>());
     const int ld = int(d.ld[L::slot]);
-    const int rr = int(d.R - d.r0), cc = int(d.C - d.c0);  // rows / cols left in the matrix
+    const int cc = int(d.C - d.c0);  // columns left in the matrix
     if constexpr (L::mode == MN) {
       // column c holds rows r0 - s_c .. r0 - s_c + TR - 1 (s_c its skew);
       // offsets from the tile's first column are 32-bit
@@ -160,13 +160,12 @@ FX_D void issue_tile(char* buf, const IssueDesc<NIN>& d) {
       constexpr int CPC = TR / W;  // chunks per column
       static_assert(NT % CPC == 0 && TC % (NT / CPC) == 0, "chunk copy shape");
       const int q = (threadIdx.x % CPC) * W;
-      const int R = int(d.R);
-      const int r0 = int(d.r0);
+      const int64_t R = d.R;  // a tile's rows may reach beyond 2^31
       const uint32_t c0 = uint32_t(d.c0);
 #pragma unroll
       for (int c = threadIdx.x / CPC; c < TC; c += NT / CPC) {
         if (c >= cc) break;
-        const int row = r0 - col_skew<W>(d.sld, d.sbase, c0 + c) + q;
+        const int64_t row = d.r0 - col_skew<W>(d.sld, d.sbase, c0 + c) + q;
         const T* s = src + (row + c * ld);
         T* t = dst + c * TR + q;
         if (row >= 0 && row + W <= R && (reinterpret_cast<uintptr_t>(s) & 15) == 0) {
@@ -185,15 +184,15 @@ FX_D void issue_tile(char* buf, const IssueDesc<NIN>& d) {
       constexpr int W = 16 / int(sizeof(T));
       constexpr int KS = NT / TC;  // stored rows per pass of the block
       static_assert(NT % TC == 0, "transposed copy shape");
-      const int rlo = int(d.r0) - (W - 1);
-      const int kb = rlo < 0 ? -rlo : 0;
-      const int left = int(d.R) - rlo;
-      const int ke = left < TR + W - 1 ? left : TR + W - 1;
+      const int64_t rlo = d.r0 - (W - 1);
+      const int kb = rlo < 0 ? int(-rlo) : 0;
+      const int64_t left = d.R - rlo;
+      const int ke = left < TR + W - 1 ? int(left) : TR + W - 1;
       const int c = threadIdx.x % TC;  // D element (c0 + c, rlo + k)
       if (c < cc) {
         int k = threadIdx.x / TC;
         if (k < kb) k += ((kb - k + KS - 1) / KS) * KS;
-        const T* s = static_cast<const T*>(d.p[L::slot]) + d.c0 + c + int64_t(rlo + k) * ld;
+        const T* s = static_cast<const T*>(d.p[L::slot]) + d.c0 + c + (rlo + k) * ld;
         T* t = dst + k * (TC + 1) + c;
         const int64_t step = int64_t(KS) * ld;
         for (; k < ke; k += KS) {
@@ -293,8 +292,7 @@ __global__ void __launch_bounds__(NT) k_batch_async(const E e, const BatchMat* _
     const char* buf = smem + b * AB;
     const int i = (threadIdx.x % RG) * V;
     const int cc = int(d.C - d.c0);
-    const int R = int(d.R);
-    const int r0 = int(d.r0);
+    const int64_t R = d.R;  // a tile's rows may reach beyond 2^31
     const uint32_t c0 = uint32_t(d.c0);
     const int ldz = int(d.ldz);
     // Z from the tile's first column on; offsets inside a matrix are 32-bit
@@ -305,7 +303,7 @@ __global__ void __launch_bounds__(NT) k_batch_async(const E e, const BatchMat* _
     for (int c = threadIdx.x / RG; c < TC; c += NT / RG) {
       if (c < cc) {
         const int sk = col_skew<W>(d.sld, d.sbase, c0 + c);
-        const int row = r0 - sk + i;  // output row of slot i
+        const int64_t row = d.r0 - sk + i;  // output row of slot i
         Pack<LL, V, CT> p;
         CT v[V];
         if (row >= 0 && row + V <= R) {  // all V slots inside the matrix
@@ -722,7 +720,8 @@ fx_status run_batch(fx_expr* x, const Root& root, int64_t n, const fx_batch_item
             lb[k].ld = m.ld[k];
           }
           if (R > 0 && C > 0 &&
-              !skew_ok<LL, T, W>(lb, has_z ? m.p[zs] : nullptr, has_z ? m.ld[zs] : 0, m.csbase, m.csld))
+              (!skew_extent(R, C) ||
+               !skew_ok<LL, T, W>(lb, has_z ? m.p[zs] : nullptr, has_z ? m.ld[zs] : 0, m.csbase, m.csld)))
             skewed = false;
         }
       }

@@ -493,8 +493,7 @@ fx_status launch_tile_skew(const Run& r, const E& e, const Slots& sl, int64_t R,
     // against 5.8 us, 501^2 7.1 against 7.9, 1001^2 8.9 against 9.2, 1561 x 1200
     // 14.2 against 10.5); FP32 is not slower at any size measured
     if (sizeof(T) == 2 && R * C < (int64_t(1) << 20) && r.tune.bps == 0) return FX_OK;
-    const int64_t lim = (int64_t(1) << 31) - 128;
-    if (R >= lim || C >= lim || !skew_ok<LL, T, V>(r.b, z, epi.ldz, sbase, sld)) return FX_OK;
+    if (!skew_extent(R, C) || !skew_ok<LL, T, V>(r.b, z, epi.ldz, sbase, sld)) return FX_OK;
     using TC_ = TileCfg<E, V>;
     constexpr int NT = skew_threads();
     auto kern = k_tile_skew<E, Epi, T, V, TC_::TR, TC_::TC, NT>;

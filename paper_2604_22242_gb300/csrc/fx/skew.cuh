@@ -344,6 +344,12 @@ bool skew_leaves(const Binding* b, int& first, uint32_t& sbase, uint32_t& sld) {
   return true;
 }
 
+// Rows and columns that the tiles can count in 32 bits: the last tile begins
+// up to a shift beyond the last row, and its end and the rows of its vectors
+// are computed too.
+constexpr int64_t kSkewExtent = (int64_t(1) << 31) - 128;
+inline bool skew_extent(int64_t R, int64_t C) { return R < kSkewExtent && C < kSkewExtent; }
+
 // Offsets inside a tile are 32-bit: leading dimensions below 2^25.
 constexpr int64_t kSkewLd = int64_t(1) << 25;
 template <class LL, int I = 0> bool skew_lds(const Binding* b) {
