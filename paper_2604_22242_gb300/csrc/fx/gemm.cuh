@@ -304,6 +304,7 @@ template <class T, int NIN, class Root> struct umma_ok {
 
 // Do two bound matrices of `es`-byte elements share memory (as whole spans)?
 inline bool overlap(const Binding& x, const Binding& y, size_t es) {
+  if (x.rows * x.cols == 0 || y.rows * y.cols == 0) return false;
   auto span = [es](const Binding& b) { return (size_t(b.ld) * size_t(b.cols - 1) + size_t(b.rows)) * es; };
   const uintptr_t p = reinterpret_cast<uintptr_t>(x.p), q = reinterpret_cast<uintptr_t>(y.p);
   return p < q + span(y) && q < p + span(x);
@@ -322,10 +323,11 @@ constexpr double kRelayoutMin = double(1 << 30), kSplitMin = double(1 << 28);
 // bases and leading dimensions; an operand without them is first copied to a
 // workspace that has (k_relayout16: 4 bytes moved per operand element, small
 // beside a large product, where the library's kernels for such operands run at
-// a fraction of the tensor cores' rate). *used is false when the shapes disagree (the caller's library
-// path reports it), for a bare or scaled product of unaligned operands
-// (nothing to fuse), when Z is written over an operand read in place beside
-// a copied one, or without workspace.
+// a fraction of the tensor cores' rate). So is, at any size, an operand that Z
+// is written over: other tiles' loads of it may come after a tile's store.
+// *used is false when the shapes disagree (the caller's library path reports
+// it), for a bare or scaled product of unaligned operands (nothing to fuse), or
+// without workspace.
 template <class T, int NIN, class Root>
 fx_status run_umma(fx_expr* x, const Root& root, cudaStream_t st, bool* used) {
   *used = false;
@@ -365,28 +367,30 @@ fx_status run_umma(fx_expr* x, const Root& root, cudaStream_t st, bool* used) {
     return encode_map<T>(m, o.p, o.rows, o.cols, o.ld, 64, mn ? 64 : box);
   };
   const bool oka = encode(&ma, a, AMN, umma::BM), okb = encode(&mb, b, BMN, pair ? umma::BN / 2 : umma::BN);
+  if ((!oka || !okb) &&
+      (ScaledProd<Root>::value || (double(M) * double(N) * double(Ka) < kRelayoutMin && x->tune.bps == 0)))
+    return FX_OK;
+  const bool mova = !oka || overlap(zb, a, sizeof(T)), movb = !okb || overlap(zb, b, sizeof(T));
   umma::Relayout ca{}, cb{};
-  if (!oka || !okb) {
-    if (ScaledProd<Root>::value || (double(M) * double(N) * double(Ka) < kRelayoutMin && x->tune.bps == 0)) return FX_OK;
-    if ((oka && overlap(zb, a, sizeof(T))) || (okb && overlap(zb, b, sizeof(T)))) return FX_OK;
+  if (mova || movb) {
     auto ldp = [](const Binding& o) { return (o.rows + 7) / 8 * 8; };
     auto bytes = [&](const Binding& o) { return (size_t(ldp(o)) * size_t(o.cols) * sizeof(T) + 255) & ~size_t(255); };
     auto copy = [&](const Binding& o, char* d) {
       const int64_t pc = (o.rows + 255) / 256;
       return umma::Relayout{o.p, d, o.rows, o.cols, o.ld, ldp(o), pc * o.cols, FastDiv::make(uint32_t(pc))};
     };
-    const size_t na = oka ? 0 : bytes(a), nb = okb ? 0 : bytes(b);
+    const size_t na = mova ? bytes(a) : 0, nb = movb ? bytes(b) : 0;
     if (x->ws_gemm.ensure(na + nb, st) != FX_OK) {
       cudaGetLastError();
       return FX_OK;
     }
     char* w = static_cast<char*>(x->ws_gemm.p);
     auto moved = [&](const Binding& o, char* d) { return Binding{d, o.rows, o.cols, ldp(o), true}; };
-    if (!oka) {
+    if (mova) {
       ca = copy(a, w);
       if (!encode(&ma, moved(a, w), AMN, umma::BM)) return FX_OK;
     }
-    if (!okb) {
+    if (movb) {
       cb = copy(b, w + na);
       if (!encode(&mb, moved(b, w + na), BMN, pair ? umma::BN / 2 : umma::BN)) return FX_OK;
     }
@@ -574,12 +578,16 @@ fx_status run_with_prods(fx_expr* x, const Root& root, int kind, cudaStream_t st
   for (int j = 0; j < n_out; ++j) bb[NIN + P + j] = x->b[NIN + j];
   size_t off = 0;
   if constexpr (ScaledProd<Root>::value) {
-    if (!unfused && kind == FX_KIND_ELEMENTWISE) {
-      using SP = ScaledProd<Root>;
-      using PT = typename SP::P;
+    using SP = ScaledProd<Root>;
+    using PT = typename SP::P;
+    using LA = Lift<decltype(PT::l), T, NIN>;
+    using RA = Lift<decltype(PT::r), T, NIN + LA::count>;
+    // straight into Z, unless Z lies over one of the last product's operands:
+    // then by way of a temporary, as for other trees
+    auto over = [&](int k) { return k < NIN && overlap(x->b[NIN], x->b[k], sizeof(T)); };
+    const bool in_place = over(Operand<typename LA::type>::slot) || over(Operand<typename RA::type>::slot);
+    if (!unfused && kind == FX_KIND_ELEMENTWISE && !in_place) {
       const PT& pr = SP::prod(root);
-      using LA = Lift<decltype(pr.l), T, NIN>;
-      using RA = Lift<decltype(pr.r), T, NIN + LA::count>;
       FX_TRY((Prods<T, NIN, std::decay_t<decltype(pr.l)>>::run(bb, pr.l, nullptr, off, true, st)));
       FX_TRY((Prods<T, NIN + LA::count, std::decay_t<decltype(pr.r)>>::run(bb, pr.r, nullptr, off,
                                                                             true, st)));
