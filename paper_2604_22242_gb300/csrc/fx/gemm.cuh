@@ -502,8 +502,11 @@ fx_status run_umma32(fx_expr* x, const Root& root, cudaStream_t st, bool* used) 
   }
   const Run r = run_of(x, st);
   unsigned int *tick = nullptr, *err = nullptr;
-  FX_TRY(tickets(r, ntiles + 2, &tick));
+  // two words and the marks of the tile rows and columns (u3::Marks), then a ticket per tile
+  const int64_t tiles_m = (M + u3::BM - 1) / u3::BM, nmarks = 2 + tiles_m + (N + shape.bn - 1) / shape.bn;
+  FX_TRY(tickets(r, nmarks + ntiles, &tick));
   FX_TRY(err_word(r, &err));
+  const u3::Marks marks{tick, tick + 2, tick + 2 + tiles_m};
   bf16* da = static_cast<bf16*>(x->ws_gemm.p);
   bf16* db = da + pa / 2;
   float* part = reinterpret_cast<float*>(db + pb / 2);
@@ -518,16 +521,16 @@ fx_status run_umma32(fx_expr* x, const Root& root, cudaStream_t st, bool* used) 
   if (!planes(a, da, AMN ? 64 : u3::BM, {u3::A1, u3::A2, u3::A3}) ||
       !planes(b, db, BMN ? 64 : shape.bn, {u3::B1, u3::B2, u3::B3}))
     return FX_OK;
-  auto split = [&](const Binding& o, bf16* d) {
+  auto split = [&](const Binding& o, bf16* d, unsigned int* m, bool mn, int tile) {
     return u3::SplitArgs{static_cast<const float*>(o.p), d, o.rows, o.cols, o.ld, ldp(o), items(o),
                          FastDiv::make(uint32_t((o.rows + 7) / 8)),
-                         aligned(o.p, 16) && o.ld % 4 == 0 ? 1 : 0};
+                         aligned(o.p, 16) && o.ld % 4 == 0 ? 1 : 0, m, mn ? 1 : 0, tile == 256 ? 8 : 7};
   };
   *used = true;
   x->last_launches = 0;
   const int64_t blocks = (items(a) + items(b) + 255) / 256;
-  u3::k_split3<<<unsigned(blocks < sms * 8 ? blocks : sms * 8), 256, 0, st>>>(split(a, da), split(b, db),
-                                                                              tick);
+  u3::k_split3<<<unsigned(blocks < sms * 8 ? blocks : sms * 8), 256, 0, st>>>(
+      split(a, da, marks.rows, AMN, u3::BM), split(b, db, marks.cols, BMN, shape.bn), marks.any);
   FX_TRY(after_launch(r, "k_split3"));
   x->last_launches = 0;  // counts launches that evaluate the tree, not those that lay out operands
   const int64_t nitems = ntiles * S;
@@ -541,11 +544,14 @@ fx_status run_umma32(fx_expr* x, const Root& root, cudaStream_t st, bool* used) 
     FX_TRY(allow_smem(kern, smem));
     kern<<<unsigned(nitems < sms ? nitems : sms), SL::THREADS, smem, st>>>(
         maps, LR::make(root), make_slots(x->b, NIN), static_cast<float*>(zb.p), zb.ld, int(M), int(N),
-        int(K), S, part, tick + 2, tick, sa, sb, err);
+        int(K), S, part, tick + nmarks, marks, sa, sb, err);
     return after_launch(r, "k_gemm_umma32");
   };
-  if (shape.bn == 256) return launch(std::integral_constant<int, 256>{});
-  return launch(std::integral_constant<int, 128>{});
+  const fx_status s = shape.bn == 256 ? launch(std::integral_constant<int, 256>{})
+                                      : launch(std::integral_constant<int, 128>{});
+  // without that kernel nothing clears the marks
+  if (s != FX_OK) cudaMemsetAsync(tick, 0, size_t(nmarks) * sizeof(unsigned int), st);
+  return s;
 }
 
 // A tree with matrix products: products into temporaries (slots NIN ..

@@ -45,8 +45,9 @@
 //
 // Operands with an infinity, a NaN, a magnitude of 2^60 or more or a nonzero
 // one below 2^-100 (its parts would be subnormal) are not computed this way:
-// k_split3 records one in a flag and every block then computes its tiles with
-// FP32 fma from the operands themselves. Below 2^60 a product is below 2^120
+// k_split3 marks the tile rows or columns of the product that one lies in, and
+// their tiles are computed after the others, with FP32 fma from the operands
+// themselves. Below 2^60 a product is below 2^120
 // and a K block's 64 of them, with the small products, below 2^127, so the
 // accumulator stays finite: a1 b2 and a2 b1 have either sign, and one of them
 // at -Inf beside a1 b1 at +Inf would give NaN where FP32 gives an infinity.
@@ -128,6 +129,8 @@ struct SplitArgs {
   int64_t items;      // 8-row pieces: ceil(d0 / 8) * d1
   FastDiv per_col;    // pieces of a column
   int vec;            // every full piece is 16-byte aligned
+  unsigned int* marks;  // the operand's tiles that hold an unsplittable value
+  int mn_rows, shift;   // tile of element (row, column): (mn_rows ? row : column) >> shift
 };
 
 // Both operands in one launch, 8 rows of a column per thread: 32 bytes read,
@@ -135,8 +138,7 @@ struct SplitArgs {
 // memory (the planes of the sizes this serves stay in L2 for the product).
 // Rows of a piece beyond d0 (ldp's padding) are written as zeros.
 static __global__ void __launch_bounds__(256) k_split3(const SplitArgs a, const SplitArgs b,
-                                                       unsigned int* flag) {
-  bool bad = false;
+                                                       unsigned int* any) {
   const int64_t n = a.items + b.items;
   for (int64_t i = int64_t(blockIdx.x) * 256 + threadIdx.x; i < n; i += int64_t(gridDim.x) * 256) {
     const bool first = i < a.items;
@@ -160,6 +162,7 @@ static __global__ void __launch_bounds__(256) k_split3(const SplitArgs a, const 
       for (int j = 0; j < 8; ++j) x[j] = r + j < o.d0 ? sload(s + j) : 0.0f;
     }
     Raw<bf16, 8> p1, p2, p3;
+    bool bad = false;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       bad |= unsplittable(x[j]);
@@ -173,8 +176,11 @@ static __global__ void __launch_bounds__(256) k_split3(const SplitArgs a, const 
     *reinterpret_cast<Raw<bf16, 8>*>(d) = p1;
     *reinterpret_cast<Raw<bf16, 8>*>(d + plane) = p2;
     *reinterpret_cast<Raw<bf16, 8>*>(d + 2 * plane) = p3;
+    if (bad) {  // every writer stores the same value
+      *any = 1u;
+      o.marks[(o.mn_rows ? r : int64_t(c)) >> o.shift] = 1u;
+    }
   }
-  if (bad) *flag = 1u;  // every writer stores the same value
 }
 
 // ---------------------------------------------------------------- product
@@ -263,69 +269,177 @@ template <int NT> FX_D bool all_of(bool v) {
   return r != 0;
 }
 
-// The product by FP32 fma from the operands themselves (unsplittable values):
-// 256 threads, 8 x 8 results each, K steps of 16 through shared memory.
+// Tiles with unsplittable values: any[0] is set when there are some, then
+// rows[tile row] and cols[tile column] hold the marks; any[1] counts blocks.
+struct Marks {
+  unsigned int *any, *rows, *cols;
+  FX_D bool direct(int tm, int tn) const { return (rows[tm] | cols[tn]) != 0u; }
+};
+
+// The product of the marked tiles by FP32 fma from the operands themselves:
+// 64 x 128 pieces, each by NG groups of 256 threads that take every NG-th K step
+// of 16 and add their sums at the end; 4 x 8 results a thread, two K steps on
+// their way by cp.async while one is multiplied from shared memory. Bound by
+// instruction issue, half of it fma, and with few marked tiles by the SMs that
+// have a piece. Microseconds with one element out of range, and with one in every
+// tile row (in brackets the loop before, which took all tiles for one element: 8
+// x 8 results by 256 threads that waited for each step's loads; then the
+// library's FP32 GEMM and the element-wise pass after it):
+//   2048 x 1536 x 2048  229, 490 (1432; 262)    1000^3          125, 103 (248; 43)
+//   3000^3              495, 1790 (4338; 840)   512 x 512 x 4096  368, 338 (974; 54)
+// (The next step held in registers instead spilled: 557 for 490; fma.rn.f32x2 was
+// no faster, 8 x 8 results by 256 threads slower.)
+template <int BN> struct Fma32 {
+  static_assert(BN == 128 || BN == 256, "one or two groups (barriers 2 and 3)");
+  static constexpr int NG = BN / 128, NT = 256 * NG;  // the block has more threads: the rest leave
+  static constexpr int RM = 4, RN = 8, TM = 16 * RM, TN = 16 * RN, KS = 16;
+  static constexpr int LA = TM + 4, LB = TN + 4;      // shared-memory rows of one k
+  static constexpr int ST = 3, STAGE = KS * (LA + LB), GROUP = ST * STAGE;
+  static constexpr int PIECES = (BM / TM) * (BN / TN);  // of a tile
+  static_assert(NG * GROUP * 4 <= int(Slots32<BN>::bytes) && (NG - 1) * TM * TN * 4 <= int(Slots32<BN>::bytes),
+                "shared memory");
+};
+// A thread's elements of a ROWS x 16 step of an operand: i = t, t + 256, ...,
+// counted along the operand's contiguous dimension.
+template <int ROWS, int LD, int STEP> struct FmaWalk {
+  static constexpr int KS = 16, N = ROWS * KS / 256;
+  const float* p;      // the first one of the next step
+  int64_t dp, dk;      // to the next one, to the next step
+  int at, da, k, kj;   // place in the staged step, its step; k of the first one and its step
+  uint32_t inside;     // bit j: row of element j is inside the operand
+  FX_D FmaWalk(const Source& s, int r0, int R, int k0, int t) {
+    const bool mn = s.s_mn == 1;
+    const int r = mn ? t % ROWS : t / KS, dr = mn ? 0 : 256 / KS;
+    k = mn ? t / ROWS : t % KS;
+    kj = mn ? 256 / ROWS : 0;
+    p = s.p + (r0 + r) * s.s_mn + (k0 + k) * s.s_k;
+    dp = dr * s.s_mn + kj * s.s_k;
+    dk = int64_t(STEP) * s.s_k;
+    at = k * LD + r;
+    da = kj * LD + dr;
+    inside = 0u;
+#pragma unroll
+    for (int j = 0; j < N; ++j) inside |= uint32_t(r0 + r + j * dr < R) << j;
+  }
+  FX_D void copy(float* step, int k0, int K) {  // zeros beyond R and K
+    const uint32_t q = tma::saddr(step + at);
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const bool in = (inside >> j & 1u) && (k0 + KS <= K || k0 + k + j * kj < K);
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(q + 4u * uint32_t(j * da)),
+                   "l"(p + j * dp), "r"(in ? 4u : 0u)
+                   : "memory");
+    }
+    p += dk;
+  }
+};
+
+// Columns n0 .. n0 + TN - 1 of rows m0 .. m0 + TM - 1 of Z.
 template <int BN, class E, int PS>
-FX_D void fma_tiles(char* smem, const E& e, const Slots& sl, float* z, int64_t ldz, int M, int N,
-                    int K, const Source& A, const Source& B, int tiles_m, int tiles_n) {
+FX_D void fma_piece(char* smem, const E& e, const Slots& sl, float* z, int64_t ldz, int M, int N,
+                    int K, const Source& A, const Source& B, int m0, int n0) {
   using LL = leaves_t<E>;
-  constexpr int KS = 16, LDS = BM + 4, NL = tl_size<LL>::value;
-  float* sa = reinterpret_cast<float*>(smem);
-  float* sb = sa + KS * LDS;
-  const int tid = threadIdx.x, tx = tid % 16, ty = (tid / 16) % 16;
-  constexpr int HALVES = BN / 128;  // 128 columns at a time
-  for (int th = blockIdx.x; th < tiles_m * tiles_n * HALVES; th += gridDim.x) {
-    int tm, tn;
-    umma::tile_of(th / HALVES, tiles_m, tiles_n, tm, tn);
-    const int m0 = tm * BM, n0 = tn * BN + th % HALVES * 128;
-    float acc[8][8];
+  using F = Fma32<BN>;
+  constexpr int NL = tl_size<LL>::value, KS = F::KS, RM = F::RM, RN = F::RN;
+  const int grp = threadIdx.x / 256, t = threadIdx.x % 256;
+  const int tx = t % 16, ty = t / 16;  // rows 4 tx .. + 3, columns 4 ty .. + 3 and 64 + 4 ty .. + 3
+  float* base = reinterpret_cast<float*>(smem) + grp * F::GROUP;
+  float* sums = reinterpret_cast<float*>(smem);
+  auto group_sync = [&]() {
+    if (grp == 0) asm volatile("bar.sync 2, 256;" ::: "memory");
+    else asm volatile("bar.sync 3, 256;" ::: "memory");
+  };
+  auto all_sync = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(F::NT) : "memory"); };
+  float acc[RM][RN];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+  for (int i = 0; i < RM; ++i)
 #pragma unroll
-      for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
-    for (int k0 = 0; k0 < K; k0 += KS) {
-      __syncthreads();
-      if (tid < 256) {
-        for (int i = tid; i < KS * BM; i += 256) {
-          // walk the operand along its contiguous dimension
-          const int ka = A.s_mn == 1 ? i / BM : i % KS, ra = A.s_mn == 1 ? i % BM : i / KS;
-          const int kb = B.s_mn == 1 ? i / BM : i % KS, rb = B.s_mn == 1 ? i % BM : i / KS;
-          sa[ka * LDS + ra] = (m0 + ra < M && k0 + ka < K)
-                                  ? sload(A.p + (m0 + ra) * A.s_mn + (k0 + ka) * A.s_k) : 0.0f;
-          sb[kb * LDS + rb] = (n0 + rb < N && k0 + kb < K)
-                                  ? sload(B.p + (n0 + rb) * B.s_mn + (k0 + kb) * B.s_k) : 0.0f;
-        }
-      }
-      __syncthreads();
-      if (tid < 256) {
-        const int kn = K - k0 < KS ? K - k0 : KS;
-        for (int k = 0; k < kn; ++k) {
-          float a[8], b[8];
+    for (int j = 0; j < RN; ++j) acc[i][j] = 0.0f;
+  const int k0 = grp * KS, steps = K > k0 ? (K - k0 + KS * F::NG - 1) / (KS * F::NG) : 0;
+  FmaWalk<F::TM, F::LA, KS * F::NG> wa(A, m0, M, k0, t);
+  FmaWalk<F::TN, F::LB, KS * F::NG> wb(B, n0, N, k0, t);
+  auto fetch = [&](int i) {  // step i, into slot i % ST
+    if (i < steps) {
+      float* step = base + i % F::ST * F::STAGE;
+      wa.copy(step, k0 + i * KS * F::NG, K);
+      wb.copy(step + KS * F::LA, k0 + i * KS * F::NG, K);
+    }
+    cpa::commit();
+  };
 #pragma unroll
-          for (int i = 0; i < 8; ++i) a[i] = sa[k * LDS + tx + 16 * i];
+  for (int i = 0; i < F::ST - 1; ++i) fetch(i);
+  for (int i = 0; i < steps; ++i) {
+    cpa::wait_pending<F::ST - 2>();
+    group_sync();  // step i has landed for all, and all have read the slot that is filled next
+    fetch(i + F::ST - 1);
+    const float* sa = base + i % F::ST * F::STAGE;
+    const float* sb = sa + KS * F::LA;
+#pragma unroll 2
+    for (int k = 0; k < KS; ++k) {  // beyond K both operands are zeros
+      const float4 a0 = *reinterpret_cast<const float4*>(sa + k * F::LA + 4 * tx);
+      const float4 b0 = *reinterpret_cast<const float4*>(sb + k * F::LB + 4 * ty);
+      const float4 b1 = *reinterpret_cast<const float4*>(sb + k * F::LB + 64 + 4 * ty);
+      const float a[RM] = {a0.x, a0.y, a0.z, a0.w}, b[RN] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-          for (int j = 0; j < 8; ++j) b[j] = sb[k * LDS + ty + 16 * j];
+      for (int i = 0; i < RM; ++i)
 #pragma unroll
-          for (int i = 0; i < 8; ++i)
+        for (int j = 0; j < RN; ++j) acc[i][j] = __fmaf_rn(a[i], b[j], acc[i][j]);
+    }
+  }
+  cpa::wait_pending<0>();
+  if (F::NG > 1) {  // group 0 adds the other group's sums
+    all_sync();     // the staged steps are read
+    if (grp > 0) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) acc[i][j] = __fmaf_rn(a[i], b[j], acc[i][j]);
+      for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < RN; ++j) sums[(i * RN + j) * 256 + t] = acc[i][j];
+    }
+    all_sync();
+    if (grp == 0) {
+#pragma unroll
+      for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < RN; ++j) acc[i][j] += sums[(i * RN + j) * 256 + t];
+    }
+  }
+  if (grp == 0) {
+#pragma unroll
+    for (int j = 0; j < RN; ++j) {
+      const int n = n0 + (j / 4) * 64 + 4 * ty + j % 4;
+#pragma unroll
+      for (int i = 0; i < RM; ++i) {
+        const int m = m0 + 4 * tx + i;
+        if (m < M && n < N) {
+          float w[NL][1];
+          umma::load_others<LL, PS, float, 1>(w, sl, m, n, 1);
+          umma::ECtx<LL, PS, float, 1> cx{w, acc[i][j], 0};
+          sstore(z + m + int64_t(n) * ldz, e.ev(cx));
         }
       }
     }
-    if (tid < 256) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int m = m0 + tx + 16 * i;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int n = n0 + ty + 16 * j;
-          if (m < M && n < N) {
-            float w[NL][1];
-            umma::load_others<LL, PS, float, 1>(w, sl, m, n, 1);
-            umma::ECtx<LL, PS, float, 1> cx{w, acc[i][j], 0};
-            sstore(z + m + int64_t(n) * ldz, e.ev(cx));
-          }
-        }
+  }
+  all_sync();  // the next piece's first step overwrites the sums
+}
+
+// Every marked tile's pieces, dealt out to the blocks in order. Each warp finds
+// the marked tiles for itself, 32 at a time.
+template <int BN, class E, int PS>
+FX_D void fma_tiles(char* smem, const E& e, const Slots& sl, float* z, int64_t ldz, int M, int N,
+                    int K, const Source& A, const Source& B, const Marks& marks, int tiles_m, int tiles_n) {
+  using F = Fma32<BN>;
+  if (threadIdx.x >= F::NT) return;
+  const int ntiles = tiles_m * tiles_n, lane = threadIdx.x % 32;
+  int64_t next = blockIdx.x, seen = 0;  // this block's next piece, pieces of the tiles so far
+  for (int base = 0; base < ntiles; base += 32) {
+    const int t = base + lane;
+    uint32_t found = __ballot_sync(0xffffffffu, t < ntiles && marks.direct(t % tiles_m, t / tiles_m));
+    for (; found != 0u; found &= found - 1u, seen += F::PIECES) {
+      const int tile = base + __ffs(int(found)) - 1;
+      for (; next < seen + F::PIECES; next += gridDim.x) {
+        const int q = int(next - seen), m0 = tile % tiles_m * BM + q % (BM / F::TM) * F::TM;
+        const int n0 = tile / tiles_m * BN + q / (BM / F::TM) * F::TN;
+        if (m0 < M && n0 < N) fma_piece<BN, E, PS>(smem, e, sl, z, ldz, M, N, K, A, B, m0, n0);
       }
     }
   }
@@ -335,7 +449,7 @@ template <int BN, bool AMN, bool BMN, class E, int PS>
 __global__ void __launch_bounds__(Slots32<BN>::THREADS, 1)
     k_gemm_umma32(const __grid_constant__ Maps maps, const E e, const Slots sl, float* z,
                   const int64_t ldz, const int M, const int N, const int K, const int S,
-                  float* part, unsigned int* tickets, unsigned int* flag, const Source srcA,
+                  float* part, unsigned int* tickets, const Marks marks, const Source srcA,
                   const Source srcB, unsigned int* err) {
   using SL = Slots32<BN>;
   extern __shared__ char smem_raw[];
@@ -347,17 +461,8 @@ __global__ void __launch_bounds__(Slots32<BN>::THREADS, 1)
   const int ntiles = tiles_m * tiles_n;
   const int nitems = ntiles * S;
   const int nk = (K + BK - 1) / BK;
-  const bool direct = __ldcg(flag) != 0u;  // the same for every thread of the grid
-  __syncthreads();
-  // the last block to have read the flag clears it (and its count) for the next launch
-  if (threadIdx.x == 0 && atomicAdd(flag + 1, 1u) == gridDim.x - 1) {
-    flag[0] = 0u;
-    flag[1] = 0u;
-  }
-  if (direct) {
-    fma_tiles<BN, E, PS>(smem, e, sl, z, ldz, M, N, K, srcA, srcB, tiles_m, tiles_n);
-    return;
-  }
+  const bool any = __ldcg(marks.any) != 0u;  // the same for every thread of the grid
+  auto direct = [&](int tm, int tn) { return any && marks.direct(tm, tn); };
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2 * NP; ++i) {
       tma::mbar_init(&bars.full[i], 1);
@@ -390,6 +495,7 @@ __global__ void __launch_bounds__(Slots32<BN>::THREADS, 1)
         const int s = it / ntiles;
         int tm, tn;
         umma::tile_of(it - s * ntiles, tiles_m, tiles_n, tm, tn);
+        if (direct(tm, tn)) continue;
         const int m0 = tm * BM, n0 = tn * BN;
         const int kb1 = int(int64_t(nk) * (s + 1) / S);
         for (int kb = int(int64_t(nk) * s / S); kb < kb1 && ok; ++kb, ++g) {
@@ -429,6 +535,11 @@ __global__ void __launch_bounds__(Slots32<BN>::THREADS, 1)
       for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
         const int s = it / ntiles;
         const int nkb = int(int64_t(nk) * (s + 1) / S) - int(int64_t(nk) * s / S);
+        if (any) {
+          int tm, tn;
+          umma::tile_of(it - s * ntiles, tiles_m, tiles_n, tm, tn);
+          if (direct(tm, tn)) continue;
+        }
         for (int kb = 0; kb < nkb && ok; ++kb, ++g) {
           const uint32_t acc = tbase + (g & 1u) * BN;
           auto ready = [&](int p) {
@@ -495,6 +606,7 @@ __global__ void __launch_bounds__(Slots32<BN>::THREADS, 1)
       bool ready = true;
       int tm, tn;
       umma::tile_of(t, tiles_m, tiles_n, tm, tn);
+      if (direct(tm, tn)) continue;
       if (s == S - 1) {
         const int i = int(threadIdx.x) - 64, n = tn * BN + i / 2;
         if (n < N) prefetch_others<leaves_t<E>, PS>(sl, int64_t(tm) * BM + (i & 1) * 64, n, M);
@@ -555,6 +667,19 @@ __global__ void __launch_bounds__(Slots32<BN>::THREADS, 1)
     fence_after();
     umma::tmem_dealloc(tbase, 2 * BN);
   }
+  if (!any) return;
+  // no copy and no product is in flight: the shared memory is free, unless a
+  // wait was given up (recorded; the result is void)
+  if (!bars.abort)
+    fma_tiles<BN, E, PS>(smem, e, sl, z, ldz, M, N, K, srcA, srcB, marks, tiles_m, tiles_n);
+  // the last block clears the marks for the next launch
+  __syncthreads();
+  if (threadIdx.x == 0) bars.last = atomicAdd(marks.any + 1, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!bars.last) return;
+  for (int i = threadIdx.x; i < tiles_m + tiles_n; i += blockDim.x)
+    (i < tiles_m ? marks.rows[i] : marks.cols[i - tiles_m]) = 0u;
+  if (threadIdx.x == 0) marks.any[0] = marks.any[1] = 0u;
 }
 
 // Tile width and K ranges per tile: the pair that minimises waves of work
