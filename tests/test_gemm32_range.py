@@ -43,3 +43,41 @@ def test_largest_finite_product(fx):
     Y = np.full((1, 129), 2.0 ** 64 * (1 - 2.0 ** -24), np.float32)
     W = np.zeros((130, 129), np.float32)
     check(evaluate(fx, X, Y, W, 2.0 ** -126), X, Y, W, 2.0 ** -126)
+
+
+def product_error(fx, X, Y):
+    """Largest error of the product in 2^-24 of |X||Y|: with W = -s X Y the
+    sigmoid's argument is s times the error, read back to 2^-25 / 2^18 of it."""
+    P = X.astype(np.float64) @ Y.astype(np.float64)
+    M = np.abs(X).astype(np.float64) @ np.abs(Y).astype(np.float64)
+    s = 2.0 ** np.floor(18 - np.log2(np.median(M)))
+    W = (-s * P).astype(np.float32)
+    z = evaluate(fx, X, Y, W, s).astype(np.float64)
+    return np.max(np.abs(np.log(z / (1 - z)) - (s * P + W)) / (s * M)) * 2 ** 24
+
+
+@pytest.mark.parametrize("k", [1, 32, 64, 300])
+def test_worst_operands_and_one_sign(fx, k):
+    """The operands whose left-out plane products are largest (2^-24 of a b),
+    and terms of one sign, whose cuts add up: four a block of at most 2 2^-24 of
+    its sum each, the small products' twenty 2^-7 of that, and a rounding a
+    block."""
+    bound = 1 + 4 * 2 + 20 * 2 / 128 + (1 + k // 64)
+    worst = np.float32(float.fromhex("0x1.00ff8p+0"))
+    assert product_error(fx, np.full((130, k), worst), np.full((k, 129), worst)) <= bound
+    rng = np.random.default_rng(8)
+    X, Y = (rng.uniform(0.01, 1, d).astype(np.float32) for d in ((200, k), (k, 150)))
+    assert product_error(fx, X, Y) <= bound
+
+
+@pytest.mark.parametrize("e", [-58, -60, -62])
+def test_small_operands(fx, e):
+    """Products near 2^-120: the parts of the operands are normal, but the
+    smallest plane products are not."""
+    rng = np.random.default_rng(9)
+    X, Y = (np.ldexp(rng.uniform(0.5, 1, d).astype(np.float32), e) for d in ((150, 300), (300, 140)))
+    W = np.full((150, 140), -0.25, np.float32)
+    s = 2.0 ** (2 * -e - 9)
+    if s >= 2.0 ** 127:
+        s = 2.0 ** 126
+    check(evaluate(fx, X, Y, W, s), X, Y, W, s)
