@@ -43,11 +43,17 @@ FX_D double m_exp(double x) { return dm::exp_fast_ok(x) ? dm::exp_fast(x) : dm::
 FX_D float m_log(float x) { return ::logf(x); }
 FX_D double m_log(double x) { return ::log(x); }
 FX_D float m_sqrt(float x) { return ::sqrtf(x); }
-FX_D double m_sqrt(double x) { return dm::sqrt_fast_ok(x) ? dm::sqrt_fast(x) : dm::sqrt_any(x); }
+FX_D double m_sqrt(double x) {
+  bool sure;
+  const double s = dm::sqrt_fast(x, sure);
+  return dm::sqrt_fast_ok(x) && sure ? s : dm::sqrt_any(x);
+}
 // Division: FP32 by the operator; FP64 by dmath.cuh
 FX_D float m_div(float a, float b) { return a / b; }
 FX_D double m_div(double a, double b) {
-  return dm::div_fast_ok(a, b) ? dm::div_fast(a, b) : dm::div_any(a, b);
+  bool sure;
+  const double s = dm::div_fast(a, b, sure);
+  return dm::div_fast_ok(a, b) && sure ? s : dm::div_any(a, b);
 }
 FX_D float m_abs(float x) { return ::fabsf(x); }
 // FP64 sign changes by integer instructions: as FP64 ones they would run at
