@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(NTC + 32) k_flat_bulk(const E e, const Slots s
     if (blockIdx.x == 0) {  // elements after the last whole 16-byte vector
       for (int64_t i = n16 + tid; i < n; i += NTC) {
         Pack<LL, 1, CT> q;
-        load_flat(q, sl, i, 0, 0, 0);
+        load_flat<false>(q, sl, i, 0, 0, 0);
         CT v1[1];
         eval_lanes<1>(e, q, v1);
         CT v[V];

@@ -129,9 +129,11 @@ template <> struct bits_as<f16> { using type = unsigned short; };
 
 // Flat layout: element i = r + c*R of every leaf. Matrix leaves are dense
 // (ld == R) and read at i; an each_col vector at r; an each_row vector at c
-// (only where V divides R, so that the V elements share one column). R is
-// passed only for trees with broadcast leaves.
-template <class LL, int V, class CT, int I = 0>
+// (only where V divides R, so that the V elements share one column). ODD: V
+// does not divide R, which counts only then. (It is tested per vector all the
+// same: with the loads in a branch, the forward of the loss at 5001 x 4999 in
+// BF16 takes 40.1 us, without 42.5.)
+template <bool ODD, class LL, int V, class CT, int I = 0>
 FX_D void load_flat(Pack<LL, V, CT>& p, const Slots& sl, int64_t i, int64_t r, int64_t c, int64_t R) {
   if constexpr (I < tl_size<LL>::value) {
     using L = typename tl_at<LL, I>::type;
@@ -143,7 +145,7 @@ FX_D void load_flat(Pack<LL, V, CT>& p, const Slots& sl, int64_t i, int64_t r, i
     if constexpr (L::mode == MN) {
       vload(dst, base + i);
     } else if constexpr (L::mode == MBC) {
-      if (V > 1 && (uint32_t(R) & uint32_t(V - 1)) != 0) {
+      if (ODD && (uint32_t(R) & uint32_t(V - 1)) != 0) {
         // the vector may run on into the next column's first rows; the
         // vector leaf is read through L1, which holds it after one column
 #pragma unroll
@@ -161,7 +163,7 @@ FX_D void load_flat(Pack<LL, V, CT>& p, const Slots& sl, int64_t i, int64_t r, i
     } else {
       dst.v[0] = sload(base + c * s.vs);
     }
-    load_flat<LL, V, CT, I + 1>(p, sl, i, r, c, R);
+    load_flat<ODD, LL, V, CT, I + 1>(p, sl, i, r, c, R);
   }
 }
 
@@ -575,8 +577,10 @@ template <class CT, bool SQRT, class S> FX_D void finish_full_reduce(S& a, const
 // ---------------------------------------------------------------- A3: flat stream
 
 // With broadcast leaves, (r, c) of element i comes from one division by R
-// per vector (FastDiv; the host guarantees n < 2^32 and R >= V).
-template <class E, class Epi, int V, int U>
+// per vector (FastDiv; the host guarantees n < 2^32 and R >= V). ODD: R is not
+// a multiple of V, a kernel of its own: the choice made per vector took the
+// forward of the loss at 8192^2 in BF16 from 67.9 to 71.2 us.
+template <class E, class Epi, int V, int U, bool ODD = false>
 __global__ void __launch_bounds__(512) k_flat(const E e, const Slots sl, const int64_t n,
                                               const Epi epi, const RedArgs red, const FastDiv fd) {
   using LL = leaves_t<E>;
@@ -606,7 +610,7 @@ __global__ void __launch_bounds__(512) k_flat(const E e, const Slots sl, const i
           c = fd.div(uint32_t(vi * V));
           r = vi * V - c * fd.d;
         }
-        load_flat(p[u], sl, vi * V, r, c, BC ? int64_t(fd.d) : 0);
+        load_flat<ODD>(p[u], sl, vi * V, r, c, ODD ? int64_t(fd.d) : 0);
       }
     }
     if constexpr (FMA64) {
@@ -647,7 +651,7 @@ __global__ void __launch_bounds__(512) k_flat(const E e, const Slots sl, const i
       }
     }
   }
-  if (V > 1 && blockIdx.x == 0) {  // the n % V trailing elements, one lane each
+  if (V > 1 && (!BC || ODD) && blockIdx.x == 0) {  // the n % V trailing elements, one lane each
     for (int64_t i = nv * V + threadIdx.x; i < n; i += bdim) {
       Pack<LL, 1, CT> q;
       int64_t r = 0, c = 0;
@@ -655,7 +659,7 @@ __global__ void __launch_bounds__(512) k_flat(const E e, const Slots sl, const i
         c = fd.div(uint32_t(i));
         r = i - c * fd.d;
       }
-      load_flat(q, sl, i, r, c, BC ? int64_t(fd.d) : 0);
+      load_flat<false>(q, sl, i, r, c, 0);
       CT v1[1];
       eval_lanes<1>(e, q, v1);
       CT v[V];

@@ -243,10 +243,13 @@ inline fx_status red_space(const Run& r, int grid, RedArgs& red) {
   return tickets(r, 1, &red.ticket);
 }
 
-template <class E, class Epi, int V, int U>
+template <class E, class Epi, int V, int U, bool ODD = false>
 fx_status launch_flat_u(const Run& r, const E& e, const Slots& sl, int64_t n, const Epi& epi,
                         RedArgs red, int64_t flat_rows) {
-  auto kern = k_flat<E, Epi, V, U>;
+  if constexpr (!ODD && V > 1 && count_mode<leaves_t<E>>(MBC) > 0) {
+    if (flat_rows % V != 0) return launch_flat_u<E, Epi, V, U, true>(r, e, sl, n, epi, red, flat_rows);
+  }
+  auto kern = k_flat<E, Epi, V, U, ODD>;
   const int block = (r.tune.block >= 64 && r.tune.block <= 512) ? r.tune.block : 256;
   const int64_t nv = n / V;
   int64_t work = (nv + int64_t(block) * U - 1) / (int64_t(block) * U);
