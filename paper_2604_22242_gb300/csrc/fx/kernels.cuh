@@ -1232,18 +1232,39 @@ FX_D void bwd_bc_finish(const GradArgs& ga, int64_t r, int64_t R, int nvalid) {
         CompSum<CT> a[V];
 #pragma unroll
         for (int j = 0; j < V; ++j) a[j].init();
-        for (int k = 0; k < ga.S; k += KU) {
-          pair_t<CT> q[KU][V];
+        if constexpr (std::is_same<CT, double>::value) {
+          // FP64 additions are scarce: none of zeros, on threads without rows or beyond
+          // the last split (64 x 64 15.9 us, 26.2 with the fixed steps below)
+          constexpr int K8 = 8 / V > 1 ? 8 / V : 1;
+          for (int k = 0; k < ga.S && nvalid > 0; k += K8) {
+            pair_t<CT> q[K8][V];
 #pragma unroll
-          for (int t = 0; t < KU; ++t)
+            for (int t = 0; t < K8; ++t)
 #pragma unroll
-            for (int j = 0; j < V; ++j)
-              q[t][j] = (k + t < ga.S && j < nvalid) ? __ldcg(part + int64_t(k + t) * R + j)
-                                                     : make_pair_of<CT>(0, 0);
+              for (int j = 0; j < V; ++j)
+                q[t][j] = (k + t < ga.S && j < nvalid) ? __ldcg(part + int64_t(k + t) * R + j)
+                                                       : make_pair_of<CT>(0, 0);
 #pragma unroll
-          for (int t = 0; t < KU; ++t)
+            for (int t = 0; t < K8; ++t)
+              if (k + t < ga.S) {
 #pragma unroll
-            for (int j = 0; j < V; ++j) a[j].merge(q[t][j].x, q[t][j].y);
+                for (int j = 0; j < V; ++j) a[j].merge(q[t][j].x, q[t][j].y);
+              }
+          }
+        } else {
+          for (int k = 0; k < ga.S; k += KU) {
+            pair_t<CT> q[KU][V];
+#pragma unroll
+            for (int t = 0; t < KU; ++t)
+#pragma unroll
+              for (int j = 0; j < V; ++j)
+                q[t][j] = (k + t < ga.S && j < nvalid) ? __ldcg(part + int64_t(k + t) * R + j)
+                                                       : make_pair_of<CT>(0, 0);
+#pragma unroll
+            for (int t = 0; t < KU; ++t)
+#pragma unroll
+              for (int j = 0; j < V; ++j) a[j].merge(q[t][j].x, q[t][j].y);
+          }
         }
 #pragma unroll
         for (int j = 0; j < V; ++j)

@@ -865,6 +865,9 @@ fx_status run_backward(fx_expr* x, const Root& root, const void* gout, void* con
       const int64_t gx = (R + int64_t(NT) * v - 1) / (int64_t(NT) * v);
       int occ = 0;
       if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, 0) != cudaSuccess || occ < 1) occ = 1;
+      // FP64: two blocks keep an SM's FP64 unit busy, and more splits only mean more
+      // FP64 work in the combine (257 x 2000: 138 us, with three blocks 178)
+      if (std::is_same<ct_of<E>, double>::value && occ > 2) occ = 2;
       const int64_t S = row_splits(gx, C, occ, U, r.tune);
       FX_TRY(space(gx, S));
       kern<<<dim3(unsigned(gx), unsigned(S)), NT, 0, st>>>(e, sl, R, C, ga);
