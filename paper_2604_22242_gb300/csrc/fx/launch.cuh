@@ -81,7 +81,10 @@ template <class K> fx_status allow_smem(K kern, int bytes) {
 // once, at least 2*minc columns per split. Rounded down: a few blocks more
 // than are resident run after all others, for as long as those did (FP64
 // maxima of the rows of 3001 x 4096: 312 blocks on 304 places took 169 us,
-// 300 take 96 us).
+// 300 take 96 us). Where S row ranges fit and S + 1 do not, two rounds of
+// C / (S + 1) columns are never fewer than one of C / S; tall matrices bear it
+// out (FP32 row maxima, rounded up and down: 40001 x 300 101 and 75 us, 45000 x
+// 2000 151 and 106, 79001 x 400 203 and 206, 200001 x 64 66.9 and 68.0).
 inline int64_t row_splits(int64_t gx, int64_t C, int occ, int minc, const Tune& t) {
   const int sms = device_sms() > 0 ? device_sms() : 1;
   const int bps = t.bps > 0 ? (t.bps < occ ? t.bps : occ) : occ;
@@ -710,6 +713,10 @@ fx_status launch_row(const Run& r, const E& e, const Slots& sl, int64_t R, int64
   // ~128 KB in flight per SM: 8 column vectors per thread for 1-2 leaves; 4
   // in FP64, whose slow arithmetic wants more warps rather than more loads each
   constexpr int NT = 256, U = !std::is_same<CT, double>::value && tl_size<LL>::value <= 2 ? 8 : 4, NS = 4;
+  // columns per split: FP64 keeps 16 with half the loads, since its combine of
+  // the splits is FP64 work too (maxima of the rows of 257 x 2000: 250 splits
+  // 42.5 us, 125 26.8), but 8 where that is all (8192 x 64 8.8 us, with 16 10.1)
+  const int minc = tl_size<LL>::value <= 2 && C > 128 ? 8 : U;
   RowRed rr{};
   rr.out = out;
   auto space = [&](int64_t gx, int64_t S) -> fx_status {
@@ -746,7 +753,7 @@ fx_status launch_row(const Run& r, const E& e, const Slots& sl, int64_t R, int64
   const int64_t gx = (R + int64_t(NT) * V - 1) / (int64_t(NT) * V);
   int occ = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, 0) != cudaSuccess || occ < 1) occ = 1;
-  const int64_t S = row_splits(gx, C, occ, U, r.tune);
+  const int64_t S = row_splits(gx, C, occ, minc, r.tune);
   FX_TRY(space(gx, S));
   kern<<<dim3(unsigned(gx > 0 ? gx : 1), unsigned(S)), NT, 0, r.st>>>(e, sl, R, C, rr);
   return after_launch(r, "k_row");
