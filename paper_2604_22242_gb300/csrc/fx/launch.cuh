@@ -684,25 +684,35 @@ fx_status launch_col(const Run& r, const E& e, const Slots& sl, int64_t R, int64
                      int64_t ldo) {
   // a warp's loads in flight cover latency with U vectors; FP64 takes fewer,
   // so that more warps (columns) fit on an SM
-  constexpr int NT = 256, U = !std::is_same<ct_of<E>, double>::value && tl_size<leaves_t<E>>::value <= 2 ? 8 : 4;
-  // blocks of two warps when a warp takes a column: with eight, the columns
-  // of 4096 filled the SMs unevenly (one round and an eighth). FP64 column
-  // sums of 3001 x 4096: 95 us with U = 8 and eight warps, 49 us so
-  constexpr int NW = 64;
+  constexpr bool dbl = std::is_same<ct_of<E>, double>::value;
+  constexpr int NT = 256, UL = tl_size<leaves_t<E>>::value <= 2 ? 8 : 4, U = dbl ? 4 : UL;
+  // blocks of two warps when a warp takes a column: with eight, the columns of
+  // 4096 filled the SMs unevenly (one round and an eighth). FP64 column sums of
+  // 3001 x 4096: 95 us with U = 8 and eight warps, 49 us so; BF16 1023 x 4000 4.2
+  // against 4.4; but FP32 1023 x 4000 4.5 with eight, 4.8 with two
+  constexpr int NW = sizeof(typename tl_at<leaves_t<E>, 0>::type::elem) == 4 ? NT : 64;
+  auto blocks = [&](auto kern) -> fx_status {
+    const int grid = grid_for(kern, NT, C > 0 ? C : 1, r.tune);
+    kern<<<grid, NT, 0, r.st>>>(e, sl, R, C, out, ldo);
+    return after_launch(r, "k_col");
+  };
   // a block per column for long FP32 columns; a warp per column otherwise,
   // and for FP64 up to 2^16 rows: its slow FP64 unit leaves a block per
   // column waiting on the block-wide merge after only a few steps
-  constexpr bool dbl = std::is_same<ct_of<E>, double>::value;
   if (R >= (dbl ? 65536 : 1024)) {
-    auto kern = k_col<E, ISMAX, V, U, NT, NT>;
-    const int grid = grid_for(kern, NT, C > 0 ? C : 1, r.tune);
-    kern<<<grid, NT, 0, r.st>>>(e, sl, R, C, out, ldo);
-  } else {
-    auto kern = k_col<E, ISMAX, V, U, 32, NW>;
-    const int64_t work = (C + NW / 32 - 1) / (NW / 32);
-    const int grid = grid_for(kern, NW, work > 0 ? work : 1, r.tune);
-    kern<<<grid, NW, 0, r.st>>>(e, sl, R, C, out, ldo);
+    if constexpr (U < UL) {
+      // the more loads in flight where all columns are resident with them:
+      // FP64 200001 x 64 167 us against 244, 160000 x 100 201 against 216, but
+      // 400 columns of 79000 206 against 119
+      auto kern = k_col<E, ISMAX, V, UL, NT, NT>;
+      if (C <= grid_for(kern, NT, int64_t(1) << 30, r.tune)) return blocks(kern);
+    }
+    return blocks(k_col<E, ISMAX, V, U, NT, NT>);
   }
+  auto kern = k_col<E, ISMAX, V, U, 32, NW>;
+  const int64_t work = (C + NW / 32 - 1) / (NW / 32);
+  const int grid = grid_for(kern, NW, work > 0 ? work : 1, r.tune);
+  kern<<<grid, NW, 0, r.st>>>(e, sl, R, C, out, ldo);
   return after_launch(r, "k_col");
 }
 
