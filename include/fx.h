@@ -232,7 +232,9 @@ fx_status fx_expr_launch_shape(const fx_expr* x, int* block, int* unroll, int* b
 /* Fixes the launch shape (what FX_TUNE_SEARCH would choose) until the next
  * fx_tune call. block: threads per block of the streaming kernels, a
  * multiple of 32 in [64, 512]; unroll: 2, 4 or 8 vectors per thread per
- * step; blocks_per_sm: 0 (as many as fit) to 32 (the shared-memory
+ * step (as many as the tree's leaves leave registers for; while no shape has
+ * been set or tuned, most dense FP64 trees take 2, not the 4 reported);
+ * blocks_per_sm: 0 (as many as fit) to 32 (the shared-memory
  * pipelines take 1 or 2); pipeline: the kernel variant.
  *   0: the library's choice per tree: tensor-map (TMA) tiles for trees
  *      with transposed leaves, bulk-copy chunks for dense trees of five or

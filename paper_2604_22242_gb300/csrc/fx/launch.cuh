@@ -337,16 +337,23 @@ fx_status launch_flat(const Run& r, const E& e, const Slots& sl, int64_t n, cons
     if (s != FX_OK || used) return s;
   }
   constexpr int UM = max_unroll<E>();
-  switch (r.tune.unroll) {
+  // Until a shape is set or tuned, FP64 trees take two vectors: they wait for
+  // the FP64 unit more than for memory, and two leave room for twice the warps.
+  // The 2-norm of 3001 x 4096 64 us against 88 with four, Z of the statistics 274
+  // against 283 (8192^2: 1451, 1442). Sums of products or squares over one or two
+  // leaves, little work per element, keep four between 2^18 and 2^21 elements,
+  // where two mean twice the blocks to combine: the 2-norm of 8192 x 64 14.2 against
+  // 16.7, of 1000 x 1000 16.7 against 18.2 (of 64 x 64 11.2 against 10.4; forward of
+  // the loss, 1000 x 1000, 38.2 against 35.5).
+  constexpr bool dbl = std::is_same<ct_of<E>, double>::value;
+  constexpr bool terms = Epi::pure_sum && (Epi::sqrt_result || prod_root<E>::value) &&
+                         tl_size<leaves_t<E>>::value <= 2;
+  const bool four = terms && n >= (int64_t(1) << 18) && n < (int64_t(1) << 21);
+  const bool two = dbl && !r.tune.tuned && !four;
+  switch (two ? 2 : r.tune.unroll) {
     case 2: return launch_flat_u<E, Epi, V, (2 < UM ? 2 : UM)>(r, e, sl, n, epi, red, flat_rows);
     case 8: return launch_flat_u<E, Epi, V, UM>(r, e, sl, n, epi, red, flat_rows);
-    default: {
-      // FP64 trees wait for the FP64 unit more than for memory, and two vectors
-      // leave room for twice the warps: the 2-norm of 3001 x 4096 64 us against
-      // 88 with four, Z of the statistics 274 against 283 (8192^2: 1451, 1442)
-      constexpr int UD = std::is_same<ct_of<E>, double>::value ? 2 : 4;
-      return launch_flat_u<E, Epi, V, (UD < UM ? UD : UM)>(r, e, sl, n, epi, red, flat_rows);
-    }
+    default: return launch_flat_u<E, Epi, V, (4 < UM ? 4 : UM)>(r, e, sl, n, epi, red, flat_rows);
   }
 }
 

@@ -25,7 +25,7 @@ struct Tune {
   int block = 256;
   int unroll = 4;
   int bps = 0;
-  bool tuned = false;
+  bool tuned = false;  // set, searched or read from the cache: honoured as it is
   // kernel variant: 0 the library's choice per tree, 1 copy pipelines
   // (cp.async tiles, bulk-copy flat chunks and rows), 2 register loads; for
   // the batched kernel, 1 selects 8-byte vectors per thread instead of 16
