@@ -491,6 +491,40 @@ fx_status launch_tile_tma(const Run& r, const E& e, const Slots& sl, int64_t R, 
   }
 }
 
+// Some transposed leaf has a leading dimension of 1 modulo V (two: modulo 4
+// only): the V-element pieces of neighbouring staged rows then begin in the same
+// banks.
+template <class LL, int M, int I = 0> bool staged_on_banks(const Binding* b) {
+  if constexpr (I < tl_size<LL>::value) {
+    using L = typename tl_at<LL, I>::type;
+    if (L::mode == MT && b[L::slot].ld % M == 1) return true;
+    return staged_on_banks<LL, M, I + 1>(b);
+  }
+  return false;
+}
+
+// Are the skewed tiles faster than one element per lane? (any size with
+// blocks_per_sm given). Microseconds, skewed against one element per lane:
+//  FP32        at every size (Z and s of 65^2 6.5, 6.8; 5003 x 4999 86, 112);
+//  2-byte      from 2^20 elements (1101^2 5.9, 8.6; 501^2 7.9, 7.1), with staging
+//              on few banks from 5 2^18 (1025^2 6.7, 5.8; 1201^2 7.7, 8.7);
+//  FP64        bound by its FP64 instructions, which the edge vectors repeat: only
+//              where a second tree is summed beside Z, from 2^19 elements and 64
+//              rows and columns (1001^2 35, 39; 257^2 14.8, 12.8; Z alone of 2049^2
+//              73, 66; 100000 x 1 24, 9);
+//  transpose-closed trees, which stage twice as much as they store: FP32 from
+//              11 2^18 elements (1701^2 13.2, 13.5; 1201^2 8.8, 8.3), FP64 never
+//              (4999^2 302, 228), 2-byte from 2^22 unless on few banks (2051^2 16.0,
+//              19.0, 4999^2 58, 98; but 3001^2 50, 34, 2301^2 24, 21).
+template <class T, class LL, bool SIDE> bool skew_pays(const Binding* b, int64_t R, int64_t C) {
+  const int64_t n = R * C, q = int64_t(1) << 18;
+  if (flip_closed<LL>())
+    return sizeof(T) == 4 ? n >= 11 * q : sizeof(T) == 2 && n >= 16 * q && !staged_on_banks<LL, 4>(b);
+  if (sizeof(T) == 8) return SIDE && n >= 2 * q && R >= 64 && C >= 64;
+  if (sizeof(T) == 2) return n >= (staged_on_banks<LL, 8>(b) ? 5 * q : 4 * q);
+  return true;
+}
+
 // k_tile_skew; *used is false when the plain leaves and Z do not share
 // their misalignment (or the leaves are of several types).
 template <class T, class E, class Epi, int V>
@@ -502,10 +536,7 @@ fx_status launch_tile_skew(const Run& r, const E& e, const Slots& sl, int64_t R,
     const void* z = nullptr;
     if constexpr (Epi::stores) z = epi.z;
     uint32_t sbase = 0, sld = 0;
-    // 2-byte types: one element per lane is faster on small matrices (49^2 4.5
-    // against 5.8 us, 501^2 7.1 against 7.9, 1001^2 8.9 against 9.2, 1561 x 1200
-    // 14.2 against 10.5); FP32 is not slower at any size measured
-    if (sizeof(T) == 2 && R * C < (int64_t(1) << 20) && r.tune.bps == 0) return FX_OK;
+    if (r.tune.bps == 0 && !skew_pays<T, LL, Epi::side_tree>(r.b, R, C)) return FX_OK;
     if (!skew_extent(R, C) || !skew_ok<LL, T, V>(r.b, z, epi.ldz, sbase, sld)) return FX_OK;
     using TC_ = TileCfg<E, V>;
     constexpr int NT = skew_threads();
@@ -528,9 +559,10 @@ fx_status launch_tile_skew(const Run& r, const E& e, const Slots& sl, int64_t R,
 // 4.0 / 6.7 / 15.4, BF16 at 2048^2 11.4 against 11.6; at 3072^2 FP32 35.6
 // against 35.9, BF16 23.6 against 19.8. Transpose-closed trees, which read
 // each element once on the TMA kernel only: 512^2 3.0 against 4.2 us, 2048^2
-// 9.8 against 9.0.
+// 9.8 against 9.0. Others with two transposed leaves: expr2 1792^2 11.8 against
+// 12.4 us, 2048^2 15.4 against 14.2.
 template <class LL> constexpr int64_t small_tiles() {
-  return flip_closed<LL>() ? int64_t(1) << 20 : int64_t(1) << 22;
+  return (flip_closed<LL>() ? int64_t(4) : count_mt<LL>() > 1 ? int64_t(15) : int64_t(16)) << 18;
 }
 
 // Tiles of a tree with transposed leaves. Launch-shape pipeline 0: the
