@@ -7,7 +7,7 @@
 // single-matrix skewed kernel (transposed leaves staged through shared
 // memory). A tree with an accu output writes one compensated partial per
 // warp of each tile; a second launch sums each matrix's partials as pairs in
-// a fixed order (one block per matrix). The list, the descriptors and both launches are
+// a fixed order. The list, the descriptors and both launches are
 // cached per item array (kept as a copy and compared whole on the next call);
 // with use_graph the launches are captured once in a CUDA graph and replayed.
 #pragma once
@@ -492,14 +492,24 @@ __global__ void __launch_bounds__(NT, skew_blocks<T>())
   }
 }
 
-// One block per matrix: its tiles' per-warp partials (nw per tile) as pairs,
-// in a fixed order (block_sum_partials). A warp per matrix took 68 us for
-// 4096 matrices of up to 8192 partials, most of it waiting for one matrix.
+// One block per matrix: its tiles' per-warp partials (nw per tile) as pairs, in
+// a fixed order; of up to kWarpPartials by one of the block's warps. A warp for
+// each of 4096 matrices of up to 8192 partials took 68 us, most of it waiting
+// for one matrix; all four warps for each of 20000 FP64 matrices of a tile or
+// two took 200 us, the FP64 additions of merging zeros.
+constexpr int64_t kWarpPartials = 256;
 template <class RT>
 __global__ void __launch_bounds__(128) k_batch_combine(const BatchMat* __restrict__ mats,
                                                        double2* part, const int sslot, const int nw) {
   const BatchMat& m = mats[blockIdx.x];
-  const double tot = block_sum_partials<RT>(pairs<RT>(part) + m.first * nw, int64_t(m.ntiles) * nw);
+  const int64_t n = int64_t(m.ntiles) * nw;
+  double tot;
+  if (n <= kWarpPartials) {  // the same for the whole block
+    if (threadIdx.x >= 32) return;
+    tot = warp_sum_partials<RT>(pairs<RT>(part) + m.first * nw, n);
+  } else {
+    tot = block_sum_partials<RT>(pairs<RT>(part) + m.first * nw, n);
+  }
   if (threadIdx.x == 0) *static_cast<RT*>(const_cast<void*>(m.p[sslot])) = RT(tot);
 }
 

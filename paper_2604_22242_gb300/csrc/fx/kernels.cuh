@@ -545,6 +545,32 @@ template <class CT> FX_D double block_sum_partials(const pair_t<CT>* part, int64
   return double(a.s) + double(a.c);
 }
 
+// The same sum by one warp, valid in lane 0. Every lane must call it.
+template <class CT> FX_D double warp_sum_partials(const pair_t<CT>* part, int64_t n) {
+  const int lane = threadIdx.x % 32;
+  CompSum<CT> a;
+  a.init();
+  for (int64_t i = lane; i < n; i += 32) {
+    const pair_t<CT> q = __ldcg(part + i);
+    a.merge(q.x, q.y);
+  }
+  warp_merge(a);
+  if constexpr (!std::is_same<CT, double>::value) {
+    if (__any_sync(0xffffffffu, redo_in_f64(a.s))) {
+      PlainSum<double> d;
+      d.init();
+      for (int64_t i = lane; i < n; i += 32) {
+        const pair_t<CT> q = __ldcg(part + i);
+        d.add(double(q.x));
+        d.add(double(q.y));
+      }
+      warp_merge(d);
+      return d.s;
+    }
+  }
+  return double(a.s) + double(a.c);
+}
+
 // Every block publishes its partial; the last one combines all of them.
 template <class CT, bool SQRT, class S> FX_D void finish_full_reduce(S& a, const RedArgs& red) {
   block_merge(a);
