@@ -212,12 +212,17 @@ fx_status fx_eval_backward(fx_expr* x, const void* grad_out, void* const* grad_p
 fx_status fx_tune(fx_expr* x, fx_tune_mode mode, void* stream);
 
 /* Autotuner of the batched entry (fx_eval_batch): times the batched
- * kernel's launch shapes - threads per block 256 or 512 (512 not for BF16 /
- * FP16), 2, 3 or 4 pipeline stages (reported as unroll 2, 4, 8), blocks per
- * SM 0 (as many as fit), 1 or 2, and the vector width each thread
- * evaluates per step (reported as pipeline 0: 16 bytes of elements, 1: 8
- * bytes) - on the given items without graph capture,
- * keeps the fastest and caches it under (expression, storage, device, n).
+ * kernels' launch shapes on the given items without graph capture, keeps
+ * the fastest and caches it under (expression, storage, device, n).
+ * Pipeline 0 is the register tiles that follow each column's misalignment,
+ * with blocks per SM 0 (as many as fit), 1 or 2 (block and unroll do not
+ * apply and stay 256 and 4); a batch with a matrix whose plain operands and
+ * Z do not share their misalignment runs the cp.async kernel instead.
+ * Pipeline 1 is the cp.async kernel with 8 bytes of elements per thread and
+ * step. The cp.async kernel is searched over threads per block 256 or 512
+ * (512 not for BF16 / FP16), 2, 3 or 4 stages (reported as unroll 2, 4, 8)
+ * and blocks per SM 0, 1 or 2. Pipeline 2, not searched, fixes the cp.async
+ * kernel with 16-byte vectors (fx_expr_set_launch_shape).
  * FX_TUNE_CACHE reads the cache; FX_TUNE_OFF restores the defaults. The
  * next fx_eval_batch uses the chosen shape (and re-captures its graph). */
 fx_status fx_tune_batch(fx_expr* x, int64_t n, const fx_batch_item* items, fx_tune_mode mode,
@@ -236,16 +241,25 @@ fx_status fx_expr_launch_shape(const fx_expr* x, int* block, int* unroll, int* b
  * been set or tuned, most dense FP64 trees take 2, not the 4 reported);
  * blocks_per_sm: 0 (as many as fit) to 32 (the shared-memory
  * pipelines take 1 or 2); pipeline: the kernel variant.
- *   0: the library's choice per tree: tensor-map (TMA) tiles for trees
- *      with transposed leaves, bulk-copy chunks for dense trees of five or
- *      more leaves, register loads otherwise;
+ *   0: the library's choice per tree and size. Trees with transposed
+ *      leaves: register tiles up to 2^22 elements (2^20 where every matrix
+ *      is read both plain and transposed, just below 2^22 for others with
+ *      two transposed leaves), tensor-map (TMA) tiles above, and
+ *      register tiles that follow each column's misalignment where TMA and
+ *      aligned vectors cannot be used but the plain operands and the output
+ *      share their misalignment, by type and size; dense trees of five or more leaves:
+ *      bulk-copy chunks; register loads otherwise. Matrix products with a
+ *      remainder: the tensor-core kernels from the sizes on where they pay.
+ *      blocks_per_sm other than 0 also asks for the TMA tiles, and for the
+ *      tensor-core kernels, at any size;
  *   1: copy pipelines wherever a tree has one: cp.async tiles for
  *      transposed leaves, bulk-copy chunks for dense trees, bulk-copy row
- *      segments for sum/max along dim 1;
- *   2: register loads everywhere.
- * A variant whose alignment rules the operands miss (TMA and bulk copies:
- * 16-byte aligned bases; TMA also leading dimensions of a multiple of 16
- * bytes) falls back to register loads. Results agree within each kernel's
+ *      segments for sum/max along dim 1; library GEMMs for products;
+ *   2: register loads everywhere; library GEMMs for products.
+ * For fx_eval_batch see fx_tune_batch. A variant whose alignment rules the
+ * operands miss (TMA and bulk copies: 16-byte aligned bases; TMA also
+ * leading dimensions of a multiple of 16 bytes) falls back to one that they
+ * meet, register loads at last. Results agree within each kernel's
  * rounding rules; the choice changes speed only.
  * FX_E_ARG for a value out of range (the shape is then unchanged). */
 fx_status fx_expr_set_launch_shape(fx_expr* x, int block, int unroll, int blocks_per_sm,

@@ -781,10 +781,10 @@ fx_status run_batch(fx_expr* x, const Root& root, int64_t n, const fx_batch_item
     }
     const E& e = inner_of(root);
     Run r = run_of(x, st);
-    // Launch shape (tunable, fx_tune_batch): threads per block 256 or 512
-    // (512 not for 2-byte types), 2, 3 or 4 pipeline stages (unroll 2, 4,
-    // 8), blocks per SM (0: as many as fit), and the vector width a thread
-    // evaluates per step (pipeline 1: 8 bytes of elements; otherwise 16).
+    // Launch shape (tunable, fx_tune_batch): blocks per SM (0: as many as fit);
+    // for the cp.async kernel threads per block 256 or 512 (512 not for 2-byte
+    // types), 2, 3 or 4 pipeline stages (unroll 2, 4, 8), and the vector width
+    // a thread evaluates per step (pipeline 1: 8 bytes of elements; otherwise 16).
     const int NTsel = (r.tune.block >= 512 && sizeof(T) != 2) ? 512 : 256;
     const int NBsel = r.tune.unroll <= 2 ? 2 : (r.tune.unroll >= 8 ? 4 : 3);
     const int VHsel = r.tune.pipe == 1 ? 1 : 0;

@@ -111,21 +111,24 @@ template <class LL, bool ALL_MIXED = false> struct SlotModes {
   }
 };
 
-// Batch autotuner: the same search over the batched kernel's launch shapes
-// (threads per block 256 / 512, 2 / 3 / 4 stages, blocks per SM, vector
-// width 16 or 8 bytes as pipeline 0 or 1), timed on the given items without
-// graph capture; cached under the batch size.
+// Batch autotuner: times the batched kernels on the given items without graph
+// capture; cached under the batch size. Pipeline 0 (16-byte vectors) with
+// blocks per SM 0, 1 and 2, and, where its kernel is the cp.async one (a matrix
+// whose operands do not share their misalignment), with 256 / 512 threads per
+// block and 2 / 3 / 4 stages too; pipeline 1 (the cp.async kernel with 8-byte
+// vectors) with all of them. Entries of a cache file written for the cp.async
+// kernel alone are under another key and not read.
 using BatchRunFn = fx_status (*)(fx_expr*, int64_t, const fx_batch_item*, cudaStream_t, int);
 inline fx_status run_tune_batch(fx_expr* x, int mode, cudaStream_t st, int64_t n,
                                 const fx_batch_item* items, BatchRunFn run) {
-  const std::string key = "batch|" + tune_key(x) + "|" + std::to_string(n);
+  const std::string key = "batch tiles|" + tune_key(x) + "|" + std::to_string(n);
   if (mode == FX_TUNE_CACHE) {
     Tune t;
     if (tune_cache_get(key, t)) x->tune = t;
     return FX_OK;
   }
   static const int blocks[] = {256, 512};
-  static const int unrolls[] = {2, 4, 8};
+  static const int unrolls[] = {4, 2, 8};
   static const int bpss[] = {0, 1, 2};
   static const int widths[] = {0, 1};
   cudaEvent_t a, b;
@@ -138,6 +141,8 @@ inline fx_status run_tune_batch(fx_expr* x, int mode, cudaStream_t st, int64_t n
   for (int bl : blocks)
     for (int un : unrolls)
       for (int bp : bpss) {
+        // the skewed kernel has one block size and no stages
+        if (vw == 0 && (bl != blocks[0] || un != unrolls[0]) && x->batch && x->batch->cur.skewed) continue;
         x->tune = Tune{bl, un, bp, true, vw};
         for (int w = 0; w < 2 && status == FX_OK; ++w) status = run(x, n, items, st, 0);
         if (status != FX_OK) break;

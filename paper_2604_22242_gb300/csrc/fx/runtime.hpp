@@ -28,7 +28,8 @@ struct Tune {
   bool tuned = false;  // set, searched or read from the cache: honoured as it is
   // kernel variant: 0 the library's choice per tree, 1 copy pipelines
   // (cp.async tiles, bulk-copy flat chunks and rows), 2 register loads; for
-  // the batched kernel, 1 selects 8-byte vectors per thread instead of 16
+  // a batch, 0 the skewed tiles where the operands allow them, 1 and 2 the
+  // cp.async kernel with 8- and 16-byte vectors per thread
   int pipe = 0;
 };
 
