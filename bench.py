@@ -88,8 +88,9 @@ TRAFFIC = {
 
 # FP64-pipe instructions per output element of FP64 trees (per lane: DFMA,
 # DADD and DMUL each take one slot): in the Z tree exp 4, sqrt 3, division 3
-# (fx/dmath.cuh), 1 + exp and the product's fma. The FP64 pipe is slower than
-# HBM on GB300.
+# (fx/dmath.cuh), 1 + exp and the product's fma; counted 12.06 with ncu
+# (smsp__inst_executed_pipe_fp64 at 3001 x 4096, 0.06 of them near ties). The
+# FP64 pipe is slower than HBM on GB300.
 FP64_PIPE_OPS = {("expr8192_f64", "Z"): 12}
 
 

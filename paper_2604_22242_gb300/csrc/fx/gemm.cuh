@@ -312,10 +312,10 @@ inline bool overlap(const Binding& x, const Binding& y, size_t es) {
 
 // Products from which copying unaligned 16-bit operands, and splitting FP32
 // ones, pays (M N K; any size with blocks_per_sm given). With the library's
-// GEMM and the pass after it on the other side: BF16 1001 x 301 x 1501 26.8
-// against 24.9 us, 513 x 7001 x 513 28.7 against 43.5, 1501^3 28.9 against
-// 61.7, 4001^3 190 against 850; FP32 257 x 3000 x 257 28.8 against 22.9,
-// 1000 x 300 x 1500 33 against 39, 1500^3 61 against 119, 3000^3 245 against
+// GEMM and the pass after it on the other side: BF16 1001 x 301 x 1501 18.4
+// against 18.3 us, 513 x 7001 x 513 22.8 against 37.3, 1501^3 25.1 against
+// 55.4, 4001^3 148 against 848; FP32 257 x 3000 x 257 28.8 against 22.9,
+// 1000 x 300 x 1500 33 against 39, 1500^3 61 against 119, 3000^3 250 against
 // 858.
 constexpr double kRelayoutMin = double(1 << 30), kSplitMin = double(1 << 28);
 // FP32 products of fewer terms keep the library's GEMM (blocks_per_sm given:

@@ -51,7 +51,7 @@
 // items to finish (a ticket; no block waits for another) adds the S partials
 // in range order and evaluates the remainder.
 //
-// Measured with sigmoid(s X Y + W) at 2048 x 1536 x 2048: 94 us (107 with
+// Measured with sigmoid(s X Y + W) at 2048 x 1536 x 2048: 93 us (107 with
 // 128-column tiles only and descriptors computed per product), against 268 us
 // for the library's FP32 GEMM and the element-wise pass after it; the
 // product's error against 64 bits is smaller (maximum of the result 8.7e-8
