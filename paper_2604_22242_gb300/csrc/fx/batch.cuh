@@ -35,11 +35,8 @@ struct BatchMat {
   int32_t skew;
   int32_t sbase;   // (first plain leaf's address / element size) mod W
 };
-struct BatchItem {
-  int32_t mat;
-  int32_t tile;
-};
-struct BatchTile {  // work item of k_batch_skew
+// A work item: tile row tr and column tc of matrix mat, for either kernel.
+struct BatchTile {
   int32_t mat, tr, tc, unused;
 };
 
@@ -105,13 +102,13 @@ template <int W> FX_D int col_skew(int64_t sld, int sbase, int64_t col) {
   return sld > 0 ? int((uint32_t(sbase) + uint32_t(col) * uint32_t(sld)) & uint32_t(W - 1)) : 0;
 }
 
-template <int NIN, int TR, int TC, int KIND, int KW>
-FX_D IssueDesc<NIN> fetch_item(const BatchMat* mats, const BatchItem* items, int64_t it,
+template <int NIN, int TR, int TC, int KIND>
+FX_D IssueDesc<NIN> fetch_item(const BatchMat* mats, const BatchTile* items, int64_t it,
                                bool valid) {
   IssueDesc<NIN> d;
   d.valid = valid ? 1 : 0;
   if (!valid) return d;
-  const BatchItem w = items[it];
+  const BatchTile w = items[it];
   const BatchMat& m = mats[w.mat];
 #pragma unroll
   for (int k = 0; k < NIN; ++k) {
@@ -122,12 +119,8 @@ FX_D IssueDesc<NIN> fetch_item(const BatchMat* mats, const BatchItem* items, int
   d.ldz = KIND != FX_KIND_FULL_REDUCE ? m.ld[NIN] : 0;
   d.R = m.rows;
   d.C = m.cols;
-  // 32-bit: a batch matrix has fewer than 2^31 tiles (64-bit division is a
-  // long instruction sequence, executed here by every thread for every item)
-  const uint32_t tiles_r = uint32_t((d.R + KW - 1 + TR - 1) / TR);  // rows plus the largest skew
-  const uint32_t tc = uint32_t(w.tile) / tiles_r;
-  d.r0 = int64_t(uint32_t(w.tile) - tc * tiles_r) * TR;
-  d.c0 = int64_t(tc) * TC;
+  d.r0 = int64_t(w.tr) * TR;
+  d.c0 = int64_t(w.tc) * TC;
   d.item = it;
   d.mat = w.mat;
   d.vec = m.vec;
@@ -248,7 +241,7 @@ FX_D void store_partial(double2* part, int64_t i, double s, double c) {
 // in 16-byte chunks of W elements.
 template <class E, class T, int TR, int TC, int NT, int NBUF, int KIND, int NIN, int VC>
 __global__ void __launch_bounds__(NT) k_batch_async(const E e, const BatchMat* __restrict__ mats,
-                                                    const BatchItem* __restrict__ items,
+                                                    const BatchTile* __restrict__ items,
                                                     const int64_t nitems, double2* part) {
   using LL = leaves_t<E>;
   using CT = ct_of<E>;
@@ -261,7 +254,7 @@ __global__ void __launch_bounds__(NT) k_batch_async(const E e, const BatchMat* _
   const int64_t G = gridDim.x;
   const int64_t mine = nitems > int64_t(blockIdx.x) ? (nitems - blockIdx.x + G - 1) / G : 0;
   auto fetch = [&](int64_t j) {
-    return fetch_item<NIN, TR, TC, KIND, W>(mats, items, blockIdx.x + j * G, j < mine);
+    return fetch_item<NIN, TR, TC, KIND>(mats, items, blockIdx.x + j * G, j < mine);
   };
   // issue a fetched item into buffer b (every thread commits a group, even an empty one)
   auto issue = [&](const IssueDesc<NIN>& d, int b) {
@@ -519,12 +512,11 @@ struct BatchCacheEntry {
   std::vector<fx_batch_item> items_seen;
   double scal_seen[FX_MAX_SCALARS] = {};
   bool built = false;
-  int pipe_seen = 0;      // launch-shape pipeline the work-list was built for
-  bool skewed = false;    // the work-list is of BatchTiles, for k_batch_skew
+  bool skewable = false;  // every matrix's operands share their misalignment
   int64_t n = 0, nitems = 0;
   Workspace dev;  // descriptors, items, partials
   BatchMat* mats = nullptr;
-  BatchItem* items = nullptr;
+  BatchTile* items = nullptr;
   double2* part = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaStream_t exec_stream = nullptr;
@@ -651,8 +643,7 @@ fx_status run_batch(fx_expr* x, const Root& root, int64_t n, const fx_batch_item
     if (!x->batch) x->batch = new (std::nothrow) BatchCache;
     if (!x->batch) return fail(FX_E_NOMEM, "out of host memory");
     BatchCacheEntry& c = x->batch->cur;
-    constexpr int STR = dbl ? 32 : 64, STC = 64;  // tiles of k_batch_skew
-    const bool same = c.built && c.mats && c.n == n && c.pipe_seen == x->tune.pipe &&
+    const bool same = c.built && c.mats && c.n == n &&
                       memcmp(c.scal_seen, x->scal, sizeof c.scal_seen) == 0 &&
                       (n == 0 || memcmp(c.items_seen.data(), items,
                                         size_t(n) * sizeof(fx_batch_item)) == 0);
@@ -669,9 +660,9 @@ fx_status run_batch(fx_expr* x, const Root& root, int64_t n, const fx_batch_item
         return items[a].rows * items[a].cols > items[b].rows * items[b].cols;
       });
       std::vector<BatchMat> mats(n);
-      std::vector<BatchItem> work;
-      std::vector<BatchTile> swork;
-      bool skewed = x->tune.pipe == 0 && V > 1 && V * sizeof(T) == 16 && tma_uniform<LL, T>();
+      std::vector<BatchTile> work;
+      std::vector<char> shifts(n, 0);  // the matrix's largest shift is known (else W - 1)
+      bool skewable = V > 1 && V * sizeof(T) == 16 && tma_uniform<LL, T>();
       for (int64_t oi = 0; oi < n; ++oi) {
         const int64_t i = order[oi];
         const fx_batch_item& it = items[i];
@@ -729,53 +720,50 @@ fx_status run_batch(fx_expr* x, const Root& root, int64_t n, const fx_batch_item
             lb[k].p = const_cast<void*>(m.p[k]);
             lb[k].ld = m.ld[k];
           }
-          if (R > 0 && C > 0 &&
-              (!skew_extent(R, C) ||
-               !skew_ok<LL, T, W>(lb, has_z ? m.p[zs] : nullptr, has_z ? m.ld[zs] : 0, m.csbase, m.csld)))
-            skewed = false;
+          if (R > 0 && C > 0) {
+            shifts[i] = skew_extent(R, C) &&
+                        skew_ok<LL, T, W>(lb, has_z ? m.p[zs] : nullptr, has_z ? m.ld[zs] : 0, m.csbase, m.csld);
+            if (!shifts[i]) skewable = false;
+          }
         }
       }
+      // One work-list for both kernels, whose tiles are the same: changing the
+      // launch shape builds and copies nothing
       for (int64_t oi = 0; oi < n; ++oi) {
         const int64_t i = order[oi];
         BatchMat& m = mats[i];
         const int64_t R = m.rows, C = m.cols;
         // row tiles cover R plus the largest shift
         constexpr int W = 16 / int(sizeof(T));
-        const int64_t tr = skewed ? (R + max_shift<W>(m.csbase, m.csld, C) + STR - 1) / STR
-                                  : (R + W - 1 + TR - 1) / TR;
-        const int64_t tc = skewed ? (C + STC - 1) / STC : (C + TCc - 1) / TCc;
+        const int shift = shifts[i] ? max_shift<W>(m.csbase, m.csld, C) : W - 1;
+        const int64_t tr = (R + shift + TR - 1) / TR, tc = (C + TCc - 1) / TCc;
         const int64_t nt = (R > 0 && C > 0) ? tr * tc : 0;
-        m.first = int64_t(skewed ? swork.size() : work.size());
+        m.first = int64_t(work.size());
         m.ntiles = int32_t(nt);
-        for (int64_t t = 0; t < nt; ++t) {
-          if (skewed) swork.push_back(BatchTile{int32_t(i), int32_t(t % tr), int32_t(t / tr), 0});
-          else work.push_back(BatchItem{int32_t(i), int32_t(t)});
-        }
+        for (int64_t t = 0; t < nt; ++t) work.push_back(BatchTile{int32_t(i), int32_t(t % tr), int32_t(t / tr), 0});
       }
-      const size_t nwork = skewed ? swork.size() : work.size();
+      const size_t nwork = work.size();
       if (c.exec) {
         cudaGraphExecDestroy(c.exec);
         c.exec = nullptr;
       }
       const size_t bm = ((sizeof(BatchMat) * n) + 255) & ~size_t(255);
-      const size_t wb = skewed ? sizeof(BatchTile) * nwork : sizeof(BatchItem) * nwork;
+      const size_t wb = sizeof(BatchTile) * nwork;
       const size_t bi = (wb + 255) & ~size_t(255);
       const size_t bp = sizeof(double2) * (NTMAX / 32) * (nwork > 0 ? nwork : 1);
       FX_TRY(c.dev.ensure(bm + bi + bp, st));
       char* base = static_cast<char*>(c.dev.p);
       c.mats = reinterpret_cast<BatchMat*>(base);
-      c.items = reinterpret_cast<BatchItem*>(base + bm);
+      c.items = reinterpret_cast<BatchTile*>(base + bm);
       c.part = reinterpret_cast<double2*>(base + bm + bi);
       if (n > 0) FX_CUDA(cudaMemcpyAsync(c.mats, mats.data(), sizeof(BatchMat) * n, cudaMemcpyHostToDevice, st));
       if (nwork > 0)
-        FX_CUDA(cudaMemcpyAsync(c.items, skewed ? static_cast<const void*>(swork.data()) : work.data(), wb,
-                                cudaMemcpyHostToDevice, st));
+        FX_CUDA(cudaMemcpyAsync(c.items, work.data(), wb, cudaMemcpyHostToDevice, st));
       FX_CUDA(cudaStreamSynchronize(st));  // host vectors die at scope end
       c.items_seen.assign(items, items + n);
       memcpy(c.scal_seen, x->scal, sizeof c.scal_seen);
       c.built = true;
-      c.skewed = skewed;
-      c.pipe_seen = x->tune.pipe;
+      c.skewable = skewable;
       c.n = n;
       c.nitems = int64_t(nwork);
     }
@@ -788,6 +776,7 @@ fx_status run_batch(fx_expr* x, const Root& root, int64_t n, const fx_batch_item
     const int NTsel = (r.tune.block >= 512 && sizeof(T) != 2) ? 512 : 256;
     const int NBsel = r.tune.unroll <= 2 ? 2 : (r.tune.unroll >= 8 ? 4 : 3);
     const int VHsel = r.tune.pipe == 1 ? 1 : 0;
+    const bool skewed = r.tune.pipe == 0 && c.skewable;
     constexpr int VW = 16 / int(sizeof(T));
     auto launch_one = [&](auto nt_c, auto nb_c) -> fx_status {
       constexpr int NT = decltype(nt_c)::value, NBUF = decltype(nb_c)::value;
@@ -817,15 +806,15 @@ fx_status run_batch(fx_expr* x, const Root& root, int64_t n, const fx_batch_item
     auto launch_skew = [&]() -> fx_status {
       if constexpr (V > 1 && V * sizeof(T) == 16 && tma_uniform<LL, T>()) {
         constexpr int KE = kind == FX_KIND_MULTI ? FX_KIND_MULTI : KIND0;
-        auto kern = k_batch_skew<E, T, V, STR, STC, SNT, KE, NIN>;
+        auto kern = k_batch_skew<E, T, V, TR, TCc, SNT, KE, NIN>;
         const int grid = grid_for(kern, SNT, c.nitems, r.tune);
-        kern<<<grid, SNT, 0, st>>>(e, c.mats, reinterpret_cast<const BatchTile*>(c.items), c.nitems, c.part);
+        kern<<<grid, SNT, 0, st>>>(e, c.mats, c.items, c.nitems, c.part);
       }
       return after_launch(r, "k_batch_skew");
     };
     auto launch_all = [&]() -> fx_status {
       if (c.nitems > 0) {
-        if (c.skewed) {
+        if (skewed) {
           FX_TRY(launch_skew());
         } else if (NTsel == 512) {
           if (NBsel == 2) FX_TRY(launch_one(I512{}, B2{}));
@@ -839,13 +828,13 @@ fx_status run_batch(fx_expr* x, const Root& root, int64_t n, const fx_batch_item
       }
       if (has_s && c.n > 0) {
         k_batch_combine<CT><<<unsigned(c.n), 128, 0, st>>>(c.mats, c.part, sslot,
-                                                           (c.skewed ? SNT : NTsel) / 32);
+                                                           (skewed ? SNT : NTsel) / 32);
         FX_TRY(after_launch(r, "k_batch_combine"));
       }
       return FX_OK;
     };
     if (!use_graph || st == nullptr) return launch_all();
-    const int shape[4] = {NTsel, NBsel, r.tune.bps, VHsel};
+    const int shape[4] = {NTsel, NBsel, r.tune.bps, skewed ? 2 : VHsel};
     if (!c.exec || c.exec_stream != st || memcmp(shape, c.exec_shape, sizeof shape) != 0) {
       if (c.exec) {
         cudaGraphExecDestroy(c.exec);

@@ -142,7 +142,7 @@ inline fx_status run_tune_batch(fx_expr* x, int mode, cudaStream_t st, int64_t n
     for (int un : unrolls)
       for (int bp : bpss) {
         // the skewed kernel has one block size and no stages
-        if (vw == 0 && (bl != blocks[0] || un != unrolls[0]) && x->batch && x->batch->cur.skewed) continue;
+        if (vw == 0 && (bl != blocks[0] || un != unrolls[0]) && x->batch && x->batch->cur.skewable) continue;
         x->tune = Tune{bl, un, bp, true, vw};
         for (int w = 0; w < 2 && status == FX_OK; ++w) status = run(x, n, items, st, 0);
         if (status != FX_OK) break;
