@@ -537,7 +537,12 @@ fx_status run_umma32(fx_expr* x, const Root& root, cudaStream_t st, bool* used) 
   const int64_t blocks = (items(a) + items(b) + 255) / 256;
   u3::k_split3<<<unsigned(blocks < sms * 8 ? blocks : sms * 8), 256, 0, st>>>(
       split(a, da, marks.rows, AMN, u3::BM), split(b, db, marks.cols, BMN, shape.bn), marks.any);
-  FX_TRY(after_launch(r, "k_split3"));
+  // without the kernel that follows nothing clears the marks
+  auto clear = [&](fx_status f) {
+    if (f != FX_OK) cudaMemsetAsync(tick, 0, size_t(nmarks) * sizeof(unsigned int), st);
+    return f;
+  };
+  FX_TRY(clear(after_launch(r, "k_split3")));
   x->last_launches = 0;  // counts launches that evaluate the tree, not those that lay out operands
   const int64_t nitems = ntiles * S;
   const u3::Source sa{static_cast<const float*>(a.p), AMN ? 1 : a.ld, AMN ? a.ld : 1};
@@ -553,11 +558,8 @@ fx_status run_umma32(fx_expr* x, const Root& root, cudaStream_t st, bool* used) 
         int(K), S, part, tick + nmarks, marks, sa, sb, err);
     return after_launch(r, "k_gemm_umma32");
   };
-  const fx_status s = shape.bn == 256 ? launch(std::integral_constant<int, 256>{})
-                                      : launch(std::integral_constant<int, 128>{});
-  // without that kernel nothing clears the marks
-  if (s != FX_OK) cudaMemsetAsync(tick, 0, size_t(nmarks) * sizeof(unsigned int), st);
-  return s;
+  return clear(shape.bn == 256 ? launch(std::integral_constant<int, 256>{})
+                               : launch(std::integral_constant<int, 128>{}));
 }
 
 // A tree with matrix products: products into temporaries (slots NIN ..
